@@ -33,6 +33,13 @@ void init_kernel_attributes();
 template <typename R>
 cudaError_t launch_zipqr(const EigDesc& e, const int* d_dims, cudaStream_t s, void* work, double* prof);
 size_t zipqr_workspace_elems(int n_max);
+size_t zipqr_group_workspace_elems(int n_max, int group_n_max);
+// planned sizes above 256: one CTA, pivoted Gram-Schmidt on G
+template <typename R>
+cudaError_t launch_zipqr_large(int n_max, const EigDesc& e, const int* d_dims, cudaStream_t s, void* work,
+                               double* prof, const EigDesc* grp, int S);
+size_t zipqr_large_workspace_elems(int n_max);
+void init_range_attributes();
 void init_qr_attributes();
 // a named truncation solver in FP64 or double-float (solver numbering of qlb_eig_check)
 cudaError_t launch_solver(bool mixed, int solver, const EigDesc& e, const int* d_dims, cudaStream_t s, void* work);

@@ -1,0 +1,214 @@
+// What the two Gram-matrix solves over a thread-block cluster share (kernels_pj.cu: the
+// truncation eigen-solve; kernels_range.cu: the zip-up range basis): access to the other
+// CTAs' shared memory, a barrier over the CTAs that work on a problem, and sums of products in
+// the working precision.
+#pragma once
+
+#include <type_traits>
+
+#include "builder.cuh"
+#include "df64.cuh"
+
+namespace qlb {
+
+namespace {
+
+constexpr int FC_NT = 256;  // threads per CTA
+constexpr int FC_NW = FC_NT / 32;
+constexpr int FC_MAX_N = 256;
+constexpr int FC_MAX_C = 16;
+// Residuals under 1e-30 of the trace (amplitudes 1e-15 of the state's) are not taken as
+// pivots: they are below what the sites hold, and FP32 seeds need their range.
+constexpr float FC_TINY = 1e-30f;
+
+template <typename R>
+struct FcEps;
+template <>
+struct FcEps<double> {
+  static constexpr double v = 2.220446049250313e-16;
+  static constexpr double pivot = 2.220446049250313e-16;
+};
+template <>
+struct FcEps<df64> {
+  static constexpr double v = 1.4210854715202004e-14;      // 2^-46: what a chain of double-float operations keeps
+  static constexpr double pivot = 3.552713678800501e-15;   // 2^-48: the significand
+};
+
+// ------------------------------------------------------------------ cluster access
+
+__device__ __forceinline__ unsigned cta_rank_in_cluster() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// address of the same shared variable in CTA `rank` of the cluster
+template <typename T>
+__device__ __forceinline__ T* on_cta(T* p, int rank) {
+  unsigned long long out;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"((unsigned long long)p), "r"(rank));
+  return (T*)out;
+}
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+// `bytes` of our shared memory at src to CTA `rank`'s at the place of dst, counted on that
+// CTA's mbarrier at the place of bar
+__device__ __forceinline__ void send_block(int rank, const void* dst, const void* src, unsigned bytes,
+                                           const unsigned long long* bar) {
+  unsigned rd, rb;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(smem_addr(dst)), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_addr(bar)), "r"(rank));
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(rd),
+               "r"(smem_addr(src)), "r"(bytes), "r"(rb)
+               : "memory");
+}
+// waits for phase `parity` of our mbarrier, a second at most; false when the wait gave up
+__device__ __forceinline__ bool bounded_wait(const unsigned long long* bar, unsigned parity) {
+  unsigned long long t0 = 0;
+  for (;;) {
+    unsigned done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (!t0) t0 = t;
+    if (t - t0 > 1000000000ull) return false;
+  }
+}
+
+// Barrier over the CTAs that work on the problem, in two halves: every CTA's mbarrier
+// counts one arrival of each of them.  Unlike the hardware's cluster barrier it leaves out
+// the CTAs that have nothing to do, and its waits are bounded.
+struct ClusterBarrier {
+  const unsigned long long* bar;
+  int ca;
+  unsigned phase;
+  bool lost;
+  __device__ __forceinline__ void arrive() {
+    __syncthreads();
+    if ((int)threadIdx.x < ca) {
+      unsigned rb;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_addr(bar)), "r"((int)threadIdx.x));
+      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rb) : "memory");
+    }
+  }
+  __device__ __forceinline__ void wait() {
+    if (!lost && !bounded_wait(bar, phase & 1)) lost = true;
+    phase++;
+  }
+};
+
+// ------------------------------------------------------------------ arithmetic
+
+__device__ __forceinline__ double pmac(double c, double a, double b) { return fma(a, b, c); }
+__device__ __forceinline__ df64 pmac(df64 c, df64 a, df64 b) { return df_mac(c, a, b); }
+__device__ __forceinline__ double pzero(double) { return 0.0; }
+__device__ __forceinline__ df64 pzero(df64) { return df64(0.f, 0.f); }
+__device__ __forceinline__ float to_f(double x) { return (float)x; }
+__device__ __forceinline__ float to_f(df64 x) { return x.hi; }
+__device__ __forceinline__ double from_f(double, float x) { return (double)x; }
+__device__ __forceinline__ df64 from_f(df64, float x) { return df64(x, 0.f); }
+
+__device__ __forceinline__ double sx(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ df64 sx(df64 v, int m) {
+  return df64(__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m));
+}
+__device__ __forceinline__ double sget(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+__device__ __forceinline__ df64 sget(df64 v, int lane) {
+  return df64(__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane));
+}
+template <typename R>
+__device__ __forceinline__ cx<R> csub_r(cx<R> a, cx<R> b) {
+  return mk<R>(a.re - b.re, a.im - b.im);
+}
+
+// 1 / sqrt(w) for w in FP32's normal range: FP32 seed y (relative error e / 2 ~ 1e-7)
+// and one third-order step, y (1 + e/2 + 3 e^2 / 8) with e = 1 - w y^2, so no division
+// or square root runs on the FP64 pipe
+__device__ __forceinline__ double rsqrt_r(double w) {
+  const double y = (double)rsqrtf((float)w);
+  const double e = fma(-w * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ df64 rsqrt_r(df64 w) {
+  const df64 y = df64(rsqrtf(w.hi), 0.f);
+  const df64 e = df_mac(df64(1.f, 0.f), -(w * y), y);
+  return df_mac(y, e * y, df64(0.5f, 0.375f * e.hi));
+}
+
+// Running sum of products.  Double-float: the high word takes a two-sum per product and
+// every error term goes to one FP32 word (Ogita, Rump & Oishi 2005, "Accurate sum and dot
+// product", Dot2 with the operands' low words), renormalised once at the end; the chain
+// from product to product is then one FP32 addition instead of a renormalised sum.
+template <typename R>
+struct Acc;
+template <>
+struct Acc<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void mac(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ void add_from(Acc o, int m) { s += __shfl_xor_sync(0xffffffffu, o.s, m); }
+};
+template <>
+struct Acc<df64> {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void mac(df64 a, df64 b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p), t;
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    df_two_sum(s, p, s, t);
+    c = __fadd_rn(c, __fadd_rn(e, t));
+  }
+  __device__ __forceinline__ df64 value() const {
+    df64 r;
+    df_two_sum(s, c, r.hi, r.lo);
+    return r;
+  }
+  // plus o of lane ^ m
+  __device__ __forceinline__ void add_from(Acc o, int m) {
+    float t;
+    const float os = __shfl_xor_sync(0xffffffffu, o.s, m), oc = __shfl_xor_sync(0xffffffffu, o.c, m);
+    df_two_sum(s, os, s, t);
+    c = __fadd_rn(__fadd_rn(c, oc), t);  // the same bits on both lanes
+  }
+};
+
+// a x + b y + c z, one renormalisation
+__device__ __forceinline__ double mul3(double a, double x, double b, double y, double c, double z) {
+  return fma(c, z, fma(b, y, a * x));
+}
+__device__ __forceinline__ df64 mul3(df64 a, df64 x, df64 b, df64 y, df64 c, df64 z) {
+  const float p1 = __fmul_rn(a.hi, x.hi), p2 = __fmul_rn(b.hi, y.hi), p3 = __fmul_rn(c.hi, z.hi);
+  const float e1 = __fmaf_rn(a.lo, x.hi, __fmaf_rn(a.hi, x.lo, __fmaf_rn(a.hi, x.hi, -p1)));
+  const float e2 = __fmaf_rn(b.lo, y.hi, __fmaf_rn(b.hi, y.lo, __fmaf_rn(b.hi, y.hi, -p2)));
+  const float e3 = __fmaf_rn(c.lo, z.hi, __fmaf_rn(c.hi, z.lo, __fmaf_rn(c.hi, z.hi, -p3)));
+  float s, t, u, v;
+  df_two_sum(p1, p2, s, t);
+  df_two_sum(s, p3, u, v);
+  df64 r;
+  df_quick_two_sum(u, __fadd_rn(__fadd_rn(e1, e2), __fadd_rn(e3, __fadd_rn(t, v))), r.hi, r.lo);
+  return r;
+}
+
+// squared norm of a column as kept beside it (FP32 pair in both forms: rotations need it
+// to FP32's relative accuracy, and its difference to another one's to the same)
+__device__ __forceinline__ df64 to_df(double x) { return df64(x); }
+__device__ __forceinline__ df64 to_df(df64 x) { return x; }
+
+// sums of two values over groups of LP lanes (LP a power of two >= 2), the first exchange
+// also splitting them over the lanes: even lanes of a group get re, odd lanes im
+template <typename R>
+__device__ __forceinline__ R csum(Acc<R> re, Acc<R> im, int LP) {
+  const bool h = threadIdx.x & 1;
+  Acc<R> q = h ? im : re;
+  q.add_from(h ? re : im, 1);
+  for (int o = 2; o < LP; o <<= 1) q.add_from(q, o);
+  return q.value();
+}
+
+}  // namespace
+
+}  // namespace qlb

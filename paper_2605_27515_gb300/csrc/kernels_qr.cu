@@ -1,4 +1,5 @@
-// Range basis of a zip-up bond without an eigen-solve.
+// Range basis of a zip-up bond without an eigen-solve, for planned sizes above 256 (up to
+// 256: kernels_range.cu, the same method over a thread-block cluster).
 //
 // The zip-up (Sec. III.A MPO.MPS product, Sec. V.A) cuts its bonds at a relative
 // weight tol * zip_tol_factor, far below the final truncation: it needs an
@@ -384,34 +385,28 @@ __global__ void __launch_bounds__(QR_NT) k_zipqr(EigDesc e, int* __restrict__ d,
 
 }  // namespace
 
-size_t zipqr_workspace_elems(int n_max) {
+size_t zipqr_large_workspace_elems(int n_max) {
   const size_t need = (size_t)n_max * n_max;
   return need * sizeof(zd) > QR_SMEM_LIMIT ? need : 1;
 }
 
+// grp: the range bases of S states' zip-up bonds in one launch (one CTA per member),
+// n_max the largest planned size over the members
 template <typename R>
-cudaError_t launch_zipqr(const EigDesc& e, const int* d_dims, cudaStream_t s, void* work, double* prof) {
-  const size_t want = (size_t)e.n_max * e.n_max * sizeof(cx<R>);
-  const int dyn = (int)(want <= QR_SMEM_LIMIT ? want : QR_SMEM_LIMIT);
-  k_zipqr<R><<<1, QR_NT, dyn, s>>>(e, (int*)d_dims, (cx<R>*)work, dyn, prof, nullptr);
-  return cudaGetLastError();
-}
-template cudaError_t launch_zipqr<double>(const EigDesc&, const int*, cudaStream_t, void*, double*);
-template cudaError_t launch_zipqr<df64>(const EigDesc&, const int*, cudaStream_t, void*, double*);
-
-// The range bases of S states' zip-up bonds in one launch (one CTA per member);
-// n_max is the largest planned size over the members.
-template <typename R>
-cudaError_t launch_zipqr_group(int n_max, const EigDesc* d_grp, int S, cudaStream_t s, double* prof) {
-  if (S <= 0) return cudaSuccess;
+cudaError_t launch_zipqr_large(int n_max, const EigDesc& e, const int* d_dims, cudaStream_t s, void* work,
+                               double* prof, const EigDesc* grp, int S) {
   const size_t want = (size_t)n_max * n_max * sizeof(cx<R>);
   const int dyn = (int)(want <= QR_SMEM_LIMIT ? want : QR_SMEM_LIMIT);
-  EigDesc dummy{};
-  k_zipqr<R, true><<<dim3(1, S), QR_NT, dyn, s>>>(dummy, nullptr, nullptr, dyn, prof, d_grp);
+  if (grp)
+    k_zipqr<R, true><<<dim3(1, S), QR_NT, dyn, s>>>(e, (int*)d_dims, (cx<R>*)work, dyn, prof, grp);
+  else
+    k_zipqr<R, false><<<1, QR_NT, dyn, s>>>(e, (int*)d_dims, (cx<R>*)work, dyn, prof, grp);
   return cudaGetLastError();
 }
-template cudaError_t launch_zipqr_group<double>(int, const EigDesc*, int, cudaStream_t, double*);
-template cudaError_t launch_zipqr_group<df64>(int, const EigDesc*, int, cudaStream_t, double*);
+template cudaError_t launch_zipqr_large<double>(int, const EigDesc&, const int*, cudaStream_t, void*, double*,
+                                                const EigDesc*, int);
+template cudaError_t launch_zipqr_large<df64>(int, const EigDesc&, const int*, cudaStream_t, void*, double*,
+                                              const EigDesc*, int);
 
 cudaError_t launch_solver(bool mixed, int solver, const EigDesc& e, const int* d_dims, cudaStream_t s, void* work) {
   if (solver == 5)
@@ -423,6 +418,7 @@ cudaError_t launch_solver(bool mixed, int solver, const EigDesc& e, const int* d
 }
 
 void init_qr_attributes() {
+  init_range_attributes();
   cudaFuncSetAttribute(k_zipqr<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QR_SMEM_LIMIT);
   cudaFuncSetAttribute(k_zipqr<df64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QR_SMEM_LIMIT);
   cudaFuncSetAttribute(k_zipqr<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QR_SMEM_LIMIT);

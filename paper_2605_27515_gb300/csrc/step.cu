@@ -1339,18 +1339,21 @@ static qlb_status group_capture(GroupExec& gx, const std::vector<qlb_state*>& ms
       if (s) return s;
     }
     if (pass == 1) break;
-    // an eigen-solve served by the kernel of a larger co-member may need more
+    // a solve served by the kernel of a larger co-member may need more
     // workspace than the member's own plan gave it: grow it, then record again
     // (the records hold the workspace pointers)
     bool grown = false;
     for (size_t p = 0; p < recs[0].size(); p++) {
-      if (recs[0][p].kind != REC_EIG) continue;
+      const int kind = recs[0][p].kind;
+      if (kind != REC_EIG && kind != REC_ZIPQR) continue;
       int gmax = 1;
       for (int m = 0; m < S; m++)
         if (p < recs[m].size()) gmax = std::max(gmax, recs[m][p].e.n_max);
       for (int m = 0; m < S; m++) {
         if (p >= recs[m].size()) continue;
-        const size_t need = eig_group_workspace_elems(recs[m][p].e.n_max, gmax);
+        const int nm = recs[m][p].e.n_max;
+        const size_t need =
+            kind == REC_EIG ? eig_group_workspace_elems(nm, gmax) : zipqr_group_workspace_elems(nm, gmax);
         if (need > ms[m]->nEw) {
           qlb_status s = realloc_buf(ctx, &ms[m]->eigw, &ms[m]->nEw, need);
           if (s) return s;
