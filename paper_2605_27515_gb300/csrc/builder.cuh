@@ -28,6 +28,12 @@ size_t eig_smem_bytes(int n_max);
 // device workspace (complex elements) the eigen-solvers need beyond shared memory
 size_t eig_workspace_elems(int n_max);
 void init_kernel_attributes();
+// planned sizes up to 256: pivoted Cholesky and one-sided Jacobi over a cluster
+bool pj_serves(int n_max);
+template <typename R>
+cudaError_t launch_pj(int n_max, const EigDesc& e, const int* d_dims, cudaStream_t s, double* prof,
+                      const EigDesc* grp = nullptr, int S = 1);
+void init_pj_attributes();
 // zip-up range basis by column-pivoted Gram-Schmidt on the Gram matrix (U and the
 // kept count as launch_eig writes them; the gate tells the Jacobi behind it to run)
 template <typename R>
@@ -54,8 +60,8 @@ size_t tc_gemm_smem_bytes();
 // member descriptors in device memory (d_grp[S]); n_max = the largest planned size
 cudaError_t launch_gemm_group(const GemmDesc* d_grp, int S, int use_df, cudaStream_t s, double* prof);
 template <typename R>
-cudaError_t launch_eig_group(int n_max, const EigDesc* d_grp, int S, cudaStream_t s, double* prof);
-size_t eig_group_workspace_elems(int n_max, int group_n_max);
+cudaError_t launch_eig_group(int n_max, int two_sided, const EigDesc* d_grp, int S, cudaStream_t s, double* prof);
+size_t eig_group_workspace_elems(int n_max, int group_n_max, int two_sided);
 template <typename R>
 cudaError_t launch_zipqr_group(int n_max, const EigDesc* d_grp, int S, cudaStream_t s, double* prof);
 void init_tc_attributes();

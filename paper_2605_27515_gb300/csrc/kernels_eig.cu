@@ -28,8 +28,8 @@
 
 #include <type_traits>
 
+#include "builder.cuh"
 #include "df64.cuh"
-#include "qlb_internal.cuh"
 
 namespace qlb {
 
@@ -985,7 +985,8 @@ size_t eig_workspace_elems(int n_max) {
 // one-CTA kernel (group_n_max <= 24 or above the cluster range) sizes its shared
 // memory for group_n_max, capped, and falls back to the member's workspace for
 // problems that do not fit; the cluster kernels need none.
-size_t eig_group_workspace_elems(int n_max, int group_n_max) {
+size_t eig_group_workspace_elems(int n_max, int group_n_max, int two_sided) {
+  if (pj_serves(group_n_max) && !two_sided) return 1;
   if (group_n_max > 24 && group_n_max <= EIG_CL_MAX_NP) return 1;
   const size_t dyn = std::min(eig_smem_bytes<double>(group_n_max), (size_t)EIG_SMEM_LIMIT);
   const int np = n_max + (n_max & 1);
@@ -1017,13 +1018,22 @@ cudaError_t launch_eig_cl(const EigDesc& e, const int* d_dims, cudaStream_t s, d
 
 template <typename R>
 cudaError_t launch_eig(const EigDesc& e, const int* d_dims, cudaStream_t s, void* work, double* prof) {
-  // Jacobi in both precisions.  The Householder + QL solve (k_heev) is not used by
+  // Up to 256: pivoted Cholesky and one-sided Jacobi (kernels_pj.cu; on GB300, cold Gram
+  // matrices of rank n with weights over 1e-12, best of three, against the two-sided solves
+  // here: FP64 n = 16 194 us against 698, n = 64 1.31 ms against 6.03, n = 128 4.21 ms
+  // against 38.8; double-float n = 16 102 us against 388, n = 64 0.69 ms against 3.83,
+  // n = 128 2.05 ms against 23.8).  The two-sided solves stay above 256, and where they are
+  // asked for as the solve of every zip-up bond: they keep directions of rounding-level
+  // weight, which the pivoted factor leaves out.
+  //
+  // Two-sided Jacobi in both precisions.  The Householder + QL solve (k_heev) is not used by
   // the step: on the literal cat_r9 map its absolute-accuracy vectors seeded a
   // blow-up that Jacobi's relative accuracy does not, and on the exactly structured
   // Gram matrices of the transmon eigenbasis (rank-one 4 x 4) it hit its iteration
   // limit with a non-finite eigenvalue; the solver sweep on GB300 (qlb_eig_check)
   // has it no faster than Jacobi above n = 8.  Planned sizes above 24: Jacobi over
   // a thread-block cluster (rows of G and V in distributed shared memory).
+  if (pj_serves(e.n_max) && !e.two_sided) return launch_pj<R>(e.n_max, e, d_dims, s, prof);
   if (e.n_max > 24 && e.n_max <= EIG_CL_MAX_NP) {
     if (e.n_max <= 128) return launch_eig_cl<R, 8>(e, d_dims, s, prof);
     return launch_eig_cl<R, 16>(e, d_dims, s, prof);
@@ -1049,8 +1059,9 @@ template cudaError_t launch_eig<df64>(const EigDesc&, const int*, cudaStream_t, 
 // the largest planned size n_max over the members (every kernel takes any runtime
 // size up to its planned one): one CTA, or one cluster, per member (blockIdx.y).
 template <typename R>
-cudaError_t launch_eig_group(int n_max, const EigDesc* d_grp, int S, cudaStream_t s, double* prof) {
+cudaError_t launch_eig_group(int n_max, int two_sided, const EigDesc* d_grp, int S, cudaStream_t s, double* prof) {
   if (S <= 0) return cudaSuccess;
+  if (pj_serves(n_max) && !two_sided) return launch_pj<R>(n_max, EigDesc{}, nullptr, s, prof, d_grp, S);
   EigDesc e{};
   e.n_max = n_max;
   if (n_max > 24 && n_max <= EIG_CL_MAX_NP) {
@@ -1068,8 +1079,8 @@ cudaError_t launch_eig_group(int n_max, const EigDesc* d_grp, int S, cudaStream_
     k_eig<R, 512, true><<<dim3(1, S), 512, dyn, s>>>(e, nullptr, nullptr, dyn, prof, d_grp);
   return cudaGetLastError();
 }
-template cudaError_t launch_eig_group<double>(int, const EigDesc*, int, cudaStream_t, double*);
-template cudaError_t launch_eig_group<df64>(int, const EigDesc*, int, cudaStream_t, double*);
+template cudaError_t launch_eig_group<double>(int, int, const EigDesc*, int, cudaStream_t, double*);
+template cudaError_t launch_eig_group<df64>(int, int, const EigDesc*, int, cudaStream_t, double*);
 
 // One named solver regardless of the size rule above (the check entry point):
 // 1 one-CTA Jacobi, 2 cluster Jacobi over 8 CTAs (n <= 128), 3 over 16 CTAs
@@ -1102,6 +1113,7 @@ template cudaError_t launch_eig_kind<double>(int, const EigDesc&, const int*, cu
 template cudaError_t launch_eig_kind<df64>(int, const EigDesc&, const int*, cudaStream_t, void*, double*);
 
 void init_kernel_attributes() {
+  init_pj_attributes();
   cudaFuncSetAttribute(k_eig<double, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIG_SMEM_LIMIT);
   cudaFuncSetAttribute(k_eig<double, 512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIG_SMEM_LIMIT);
   cudaFuncSetAttribute(k_eig<df64, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIG_SMEM_LIMIT);

@@ -148,6 +148,7 @@ struct EigDesc {
   DimExpr cap;       // cap on k
   double gap;        // degeneracy gap
   int max_sweeps;
+  int two_sided;     // 1: two-sided Jacobi at every size (the solve of every zip-up bond)
   double* kept_weight;  // optional: sum of kept eigenvalues
   double* total_weight; // optional: sum of all eigenvalues
   double* disc_stat;    // optional: running max of discarded relative weight

@@ -1016,6 +1016,7 @@ qlb_status enqueue_step(qlb_state* st, const Kraus& K, bool count_step) {
     e.gap = o.degeneracy_gap;
     e.max_sweeps = o.max_sweeps;
     e.err = st->d_err;
+    e.two_sided = !o.zip_solver;
     if ((s = zip_range(st, e))) return s;
     // carry C' = U^dag M  -> [k][(r, b)]
     g = gdesc();
@@ -1353,7 +1354,8 @@ static qlb_status group_capture(GroupExec& gx, const std::vector<qlb_state*>& ms
         if (p >= recs[m].size()) continue;
         const int nm = recs[m][p].e.n_max;
         const size_t need =
-            kind == REC_EIG ? eig_group_workspace_elems(nm, gmax) : zipqr_group_workspace_elems(nm, gmax);
+            kind == REC_EIG ? eig_group_workspace_elems(nm, gmax, recs[m][p].e.two_sided)
+                            : zipqr_group_workspace_elems(nm, gmax);
         if (need > ms[m]->nEw) {
           qlb_status s = realloc_buf(ctx, &ms[m]->eigw, &ms[m]->nEw, need);
           if (s) return s;
@@ -1450,8 +1452,8 @@ static qlb_status group_capture(GroupExec& gx, const std::vector<qlb_state*>& ms
                   : launch_zipqr_group<double>(n_max, (const EigDesc*)t, S, gs, nullptr);
         break;
       case REC_EIG:
-        e = r0.df ? launch_eig_group<df64>(n_max, (const EigDesc*)t, S, gs, nullptr)
-                  : launch_eig_group<double>(n_max, (const EigDesc*)t, S, gs, nullptr);
+        e = r0.df ? launch_eig_group<df64>(n_max, r0.e.two_sided, (const EigDesc*)t, S, gs, nullptr)
+                  : launch_eig_group<double>(n_max, r0.e.two_sided, (const EigDesc*)t, S, gs, nullptr);
         break;
     }
   }
