@@ -30,10 +30,17 @@
 // CTA holds two blocks, rotates the b x b pairs between them (in its first turn of a
 // sweep also the pairs inside each block) with one barrier per round of b pairs, then
 // hands the blocks on in the round-robin order of Brent & Luk (1985) through
-// distributed shared memory: 2 C - 1 cluster barriers per sweep.  In the
+// distributed shared memory: 2 C - 1 exchanges per sweep.  In the
 // factorisation a CTA holds n / C rows, one cluster barrier per pivot.  C follows the
 // run-time size (pj_ctas), so that a problem takes the same split, and gives the same
 // bits, whatever larger size it was launched for; CTAs beyond C leave at once.
+//
+// Measured on GB300, cold Gram matrices of rank n with weights over 1e-12 (against the
+// two-sided Jacobi solves of kernels_eig.cu): FP64 n = 16 194 us (698), n = 32 460 us
+// (1,925), n = 64 1.31 ms (6.03), n = 128 4.21 ms (38.8); double-float n = 16 102 us (388),
+// n = 32 266 us (1,251), n = 64 0.69 ms (3.83), n = 128 2.05 ms (23.8).  At n = 64 an FP64 round of
+// four pairs to a CTA takes 4,700 cycles, ~3,500 of them the FP64 pipe; a double-float
+// round 2,100, the latency of its chain.
 //
 // R = double (the FP64 form) or df64 (the mixed forms); G and the vectors are FP64.
 
@@ -53,9 +60,9 @@ constexpr int PJ_SLOTS = PJ_MAX_N + 2 * PJ_MAX_C;  // columns with the padding o
 
 // CTAs that work on a problem of size n (a power of two).  An FP64 round costs its ~50
 // warp-wide instructions at 64 clocks whatever its pairs, so four pairs to a CTA (one warp to
-// each partition) is the fastest split until the 16 CTAs of a cluster run out; in double-float
-// small problems lose more to the exchange (~2,000 cycles) than they gain by it: n = 24
-// 206 us on one CTA, 258 us on four.
+// each partition) is the fastest split until the 16 CTAs of a cluster run out.  In
+// double-float a round of n = 24 takes 2,600 cycles on one CTA and an exchange of blocks
+// 2,000, so small problems stay on one.
 template <typename R>
 __host__ __device__ inline int pj_ctas(int n) {
   if (std::is_same<R, double>::value) return n <= 8 ? 1 : n <= 16 ? 2 : n <= 32 ? 4 : n <= 64 ? 8 : 16;
