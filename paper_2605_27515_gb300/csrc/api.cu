@@ -459,7 +459,7 @@ static qlb_status mpo_to_dense(qlb_ctx* ctx, const Mpo& W, double* out, size_t n
     g.m_max = (int)rows;
     g.n_max = (int)nn;
     g.nb_max = 1;
-    QLB_CUDA_TRY(launch_gemm<double>(g, nullptr, ctx->stream, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, nullptr, ctx->stream, nullptr));
     dev_free(ctx, T);
     T = nT;
     rows *= 4;
@@ -540,7 +540,7 @@ QLB_API qlb_status qlb_state_to_dense(qlb_state* st, double* out, size_t n_doubl
     g.m_max = (int)rows;
     g.n_max = (int)nn;
     g.nb_max = 1;
-    QLB_CUDA_TRY(launch_gemm<double>(g, nullptr, st->stream, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, nullptr, st->stream, nullptr));
     dev_free(ctx, T);
     T = nT;
     rows *= 2;
@@ -768,7 +768,7 @@ QLB_API qlb_status qlb_purity(qlb_state* st, double* out) {
   g.alpha_re = 1;
   g.m_max = g.n_max = mu;
   g.nb_max = 1;
-  QLB_CUDA_TRY(launch_gemm<double>(g, nullptr, st->stream, nullptr));
+  QLB_CUDA_TRY(launch_gemm(g, nullptr, st->stream, nullptr));
   k_sum_abs2_n<<<1, 256, 0, st->stream>>>(G, (long)mu * mu, acc);
   double h = 0, tr = 0;
   QLB_CUDA_TRY(cudaMemcpyAsync(&h, acc, sizeof(double), cudaMemcpyDeviceToHost, st->stream));
@@ -1182,7 +1182,7 @@ QLB_API qlb_status qlb_zgemm_check(int device, int engine, int m, int n, int k, 
   float t = 0.f;
   for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {
     cudaEventRecord(e0, 0);
-    e = engine == 2 ? launch_gemm_tc(g, nullptr, 0, derr, nullptr) : launch_gemm<double>(g, nullptr, 0, nullptr);
+    e = engine == 2 ? launch_gemm_tc(g, nullptr, 0, derr, nullptr) : launch_gemm(g, nullptr, 0, nullptr);
     cudaEventRecord(e1, 0);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     if (e == cudaSuccess) cudaEventElapsedTime(&t, e0, e1);

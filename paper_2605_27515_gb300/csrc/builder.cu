@@ -716,7 +716,7 @@ qlb_status mpo_compress(qlb_ctx* ctx, Mpo& W, double tol, int cap) {
     g.m_max = k;
     g.n_max = n2;
     g.nb_max = 1;
-    QLB_CUDA_TRY(launch_gemm<double>(g, nullptr, s, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, nullptr, s, nullptr));
     dev_free(ctx, W.core[i + 1]);
     dev_free(ctx, Rr);
     W.core[i + 1] = nc;
@@ -749,7 +749,7 @@ qlb_status mpo_compress(qlb_ctx* ctx, Mpo& W, double tol, int cap) {
     g.m_max = m2;
     g.n_max = k;
     g.nb_max = 1;
-    QLB_CUDA_TRY(launch_gemm<double>(g, nullptr, s, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, nullptr, s, nullptr));
     dev_free(ctx, W.core[i - 1]);
     dev_free(ctx, US);
     W.core[i - 1] = nc;
@@ -797,7 +797,7 @@ qlb_status dense_mul(qlb_ctx* ctx, const zd* A, int opA, const zd* B, int N, zd*
   g.alpha_re = 1;
   g.m_max = g.n_max = N;
   g.nb_max = 1;
-  QLB_CUDA_TRY(launch_gemm<double>(g, nullptr, ctx->stream, nullptr));
+  QLB_CUDA_TRY(launch_gemm(g, nullptr, ctx->stream, nullptr));
   return QLB_OK;
 }
 

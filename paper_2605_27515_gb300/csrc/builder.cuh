@@ -13,10 +13,9 @@ qlb_status dev_alloc(qlb_ctx* ctx, void** p, size_t bytes);
 void dev_free(qlb_ctx* ctx, void* p);
 std::map<void*, std::pair<size_t, qlb_ctx*>>& g_alloc_sizes();
 
-template <typename R>
 cudaError_t launch_gemm(const GemmDesc& g, const int* d_dims, cudaStream_t s, double* prof);
 // workspace of the work-distributed GEMM for a grid of `grid` CTAs (complex elements;
-// its counters must start at zero), and the default grid (two CTAs per SM)
+// its counters must start at zero), and the default grid (four CTAs per SM)
 size_t gemm_workspace_elems(int grid);
 int gemm_grid_default();
 template <typename R>

@@ -1,20 +1,27 @@
-// Batched complex GEMM of the step whose shapes are read from device memory,
-// templated on the real type (double for the FP64 form, float for FP32 parts).
+// Batched complex GEMM of the step whose shapes are read from device memory, in FP64 or,
+// for the mixed forms, multiplied and summed in double-float with FP64 operands and results.
 //
 // The step's GEMMs are small and their sizes change every step (bond dimensions
 // live in device memory), while the launch configuration is fixed when the step is
-// captured as a CUDA graph.  On this GPU one SM retires ~2 FP64 FMAs per clock, so
-// a GEMM whose 32 x 32 output tiles cover only a few SMs runs at a few percent of
-// the chip.  The kernel is therefore persistent over a fixed grid (two CTAs per SM
-// when a workspace is given) and decides the decomposition at run time from the
-// actual sizes: with T output tiles and G CTAs it splits the K range into
-// s = min(G / T, ceil(K / 16), cap) parts, so that T * s work items keep the SMs
-// busy.  Each (tile, part) item writes its partial tile to the workspace; the CTA
-// that finishes a tile last (a per-tile counter, no waiting) adds the s partials in
-// part order and applies alpha and beta, so the result does not depend on timing.
+// captured as a CUDA graph.  On this GPU one SM retires ~2 FP64 FMAs per clock, so what
+// counts is how evenly the products are spread over the SMs: a 32 x 32 x 16 block of
+// complex products takes one SM 16 us, a 16 x 16 x 16 block 4 us, an 8 x 8 x 16 block 1 us.
+// The kernel is persistent over a fixed grid (four CTAs per SM) and decides the
+// decomposition at run time from the actual sizes: output tiles of 16 x 16 or 8 x 8 (the
+// eight warps of a CTA take a quarter of the K chunk each), whichever finishes first with
+// its padding counted, and, with a workspace, a split of the K range into s parts while
+// tiles are fewer than CTAs and a part still outweighs what adding the parts costs.  Each
+// (tile, part) item writes its partial tile to the workspace; the CTA that finishes a
+// tile last (a per-tile counter, no waiting) adds the s partials in part order and applies
+// alpha and beta, so the result does not depend on timing.
+//
+// Measured on GB300 (C = A B, m x n x k; before: 32 x 32 tiles on two CTAs per SM, parts of 16
+// upwards): FP64 16 x 16 x 16 9 us (16), 20 x 32 x 14 9 us (19), 30 x 30 x 30 10 us (28),
+// 64^3 12 us (30), 60 x 60 x 2600 104 us (166), 128 x 128 x 600 103 us (100, of which the FP64
+// pipe needs 62); double-float 9 us (13), 8 us (16), 9 us (22), 11 us (21), 62 us (91), 55 us (52).
+// What is left of the small ones is the launch and a chain of three trips to L2.
 
 #include <algorithm>
-#include <cfloat>
 #include <type_traits>
 
 #include "df64.cuh"
@@ -24,243 +31,289 @@ namespace qlb {
 
 namespace {
 
-constexpr int GB_M = 32, GB_N = 32, GB_K = 16, G_THREADS = 256;
-constexpr int GB_TILE = GB_M * GB_N;
-constexpr int GB_SPLIT_CAP = 64;  // default cap on the K split
+constexpr int G_THREADS = 256;
+constexpr int GB_K = 32;                  // K chunk in shared memory
+constexpr int GB_TILE = 16 * 16;          // entries of a partial tile in the workspace
+constexpr int GB_SPLIT_CAP = 64;          // default cap on the K split
+constexpr int GB_SMEM = 2 * GB_K * 17;    // operand chunks (complex entries)
 
-template <typename R>
-__device__ __forceinline__ cx<R> ldop(const cx<R>* P, int op, long ld, int i, int k) {
-  // element (i, k) of op(P)
-  if (op == OP_N) return P[(long)i * ld + k];
-  cx<R> v = P[(long)k * ld + i];
-  if (op == OP_C) v.im = -v.im;
-  return v;
+// FP64 -> double-float without the FP64 pipe: hi is the high half of the significand
+// rounded to nearest (an integer addition on the bit pattern carries into the exponent as
+// rounding should), lo the signed rest, an integer below 2^28 units of the last place.
+// Values outside FP32's range for either half take the conversions (out of line: inlined,
+// the compiler executes them for every value beside the selection, on the FP64 pipe).
+__device__ __noinline__ df64 split_df_slow(double x) { return df64(x); }
+__device__ __forceinline__ df64 split_df(double x) {
+  const long long u = __double_as_longlong(x);
+  const long long mag = u & 0x7fffffffffffffffll;
+  const int e = (int)(mag >> 52);
+  if (mag == 0) return df64(0.f, 0.f);
+  if (e < 1023 - 73 || e > 1023 + 126) return split_df_slow(x);
+  const long long hb = (mag + (1ll << 28)) & ~((1ll << 29) - 1);
+  const int rest = (int)(mag - hb);
+  const unsigned sign = (unsigned)((unsigned long long)u >> 32) & 0x80000000u;
+  const float hi = __uint_as_float(((unsigned)(hb >> 29) - ((1023u - 127u) << 23)) | sign);
+  const float ulp = __uint_as_float(((unsigned)(e - 1023 - 52 + 127) << 23) | sign);
+  return df64(hi, __fmul_rn(__int2float_rn(rest), ulp));
 }
+__device__ __forceinline__ cx<double> to_c(cx<double>*, zd v) { return v; }
+__device__ __forceinline__ cx<df64> to_c(cx<df64>*, zd v) { return mk<df64>(split_df(v.re), split_df(v.im)); }
 
-// storage -> compute type of an operand, compute -> storage type of a result
-template <typename C, typename S>
-__device__ __forceinline__ cx<C> to_c(cx<S> v) {
-  return mk<C>(C(v.re), C(v.im));
-}
-template <typename S, typename C>
-__device__ __forceinline__ cx<S> to_s(cx<C> v) {
-  return mk<S>((S)v.re, (S)v.im);
-}
 // a partial tile entry written by another CTA of this launch (past L1)
-__device__ __forceinline__ cx<double> ldcg_cx(const cx<double>* p) { return mk<double>(__ldcg(&p->re), __ldcg(&p->im)); }
-__device__ __forceinline__ cx<float> ldcg_cx(const cx<float>* p) { return mk<float>(__ldcg(&p->re), __ldcg(&p->im)); }
+__device__ __forceinline__ cx<double> ldcg_cx(const cx<double>* p) {
+  const double2 v = __ldcg((const double2*)p);
+  return mk<double>(v.x, v.y);
+}
 __device__ __forceinline__ cx<df64> ldcg_cx(const cx<df64>* p) {
   const float4 v = __ldcg((const float4*)p);
   return mk<df64>(df64(v.x, v.y), df64(v.z, v.w));
 }
-// acc += a * b
-template <typename C>
-__device__ __forceinline__ void cmac(cx<C>& acc, cx<C> a, cx<C> b) {
-  cfma(acc, a, b);
-}
-template <>
-__device__ __forceinline__ void cmac<df64>(cx<df64>& acc, cx<df64> a, cx<df64> b) {
-  acc.re = df_mac(acc.re, a.re, b.re);
-  acc.re = df_mac(acc.re, -a.im, b.im);
-  acc.im = df_mac(acc.im, a.re, b.im);
-  acc.im = df_mac(acc.im, a.im, b.re);
-}
 
-template <typename R>
-__device__ __forceinline__ cx<R> gemm_alpha(const GemmDesc& g) {
-  cx<R> alpha = mk<R>((R)g.alpha_re, (R)g.alpha_im);
+// Running sum of products.  Double-float: a two-sum of each product into the high word, its
+// error terms into one FP32 word, renormalised every second product (settle): the chain
+// from product to product is one FP32 addition, and the error word stays at the rounding
+// level of the sum.
+template <typename C>
+struct GAcc;
+template <>
+struct GAcc<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void mac(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ void settle() {}
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct GAcc<df64> {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void mac(df64 a, df64 b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p), t;
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    df_two_sum(s, p, s, t);
+    c = __fadd_rn(c, __fadd_rn(e, t));
+  }
+  __device__ __forceinline__ void settle() { df_quick_two_sum(s, c, s, c); }
+  __device__ __forceinline__ df64 value() const {
+    df64 r;
+    df_two_sum(s, c, r.hi, r.lo);
+    return r;
+  }
+};
+
+__device__ __forceinline__ zd gemm_alpha(const GemmDesc& g) {
+  zd alpha = mk<double>(g.alpha_re, g.alpha_im);
   if (g.alpha_scale) {
     double s = *g.alpha_scale;
     if (g.alpha_scale_rsqrt) s = (s > 0.0) ? 1.0 / sqrt(s) : 0.0;
-    alpha = cscale(alpha, (R)s);
+    alpha = cscale(alpha, s);
   }
   return alpha;
 }
 
-// R: the storage type of A, B, C; Cm: the type the products are formed and summed in
-// (R itself, or double-float for FP64 storage in the mixed forms)
-template <typename R, typename Cm, bool GRP>
-__global__ void __launch_bounds__(G_THREADS) k_gemm(const GemmDesc g_in, const int* __restrict__ d_in, double* prof,
-                                                    const GemmDesc* __restrict__ grp) {
+// cycles that one SM spends on a K of `k` for one tile of TS x TS outputs: ~2 per complex
+// product in FP64 (four FMAs at two per clock), ~0.4 in double-float (~50 FP32
+// instructions at 128 lanes), and what an item costs besides
+template <typename Cm>
+__device__ __forceinline__ float tile_cycles(int ts, int k) {
+  return (std::is_same<Cm, double>::value ? 2.0f : 0.4f) * (float)(ts * ts) * (float)k +
+         600.f;
+}
+
+struct GemmPlan {
+  int m, n, K, nb1, nb2;
+  int tm, tn, ks, chunk;
+  long ntiles;
+};
+
+// One launch's work items with TS x TS tiles.
+template <typename Cm, int TS>
+__device__ void gemm_items(const GemmDesc& g, const int* __restrict__ d, const GemmPlan& P, int gnom, unsigned char* sm,
+                          int* s_last) {
+  constexpr int SL = G_THREADS / (TS * TS);  // K slices of a chunk (1 or 4)
+  constexpr int LD = TS + 1;
+  constexpr int NL = TS * GB_K / G_THREADS;  // loads per thread and operand
+  cx<Cm>* As = (cx<Cm>*)sm;                  // [k][row]
+  cx<Cm>* Bs = As + GB_K * LD;               // [k][column]
+  const int tid = threadIdx.x;
+  const int slice = tid / (TS * TS), o = tid % (TS * TS);
+  const int tx = o % TS, ty = o / TS;
+  const int lda = dev_eval(g.lda, d), ldb = dev_eval(g.ldb, d);
+  cx<Cm>* part_ws = (cx<Cm>*)g.ws;
+  int* counters = g.ws ? (int*)(part_ws + (long)gnom * GB_TILE) : nullptr;
+  const long items = P.ntiles * P.ks;
+  for (long it = blockIdx.x; it < items; it += gridDim.x) {
+    const long tile = it / P.ks;
+    const int kp = (int)(it - tile * P.ks);
+    const int bz = (int)(tile / ((long)P.tm * P.tn));
+    const int t2 = (int)(tile - (long)bz * P.tm * P.tn);
+    const int row0 = (t2 / P.tn) * TS, col0 = (t2 % P.tn) * TS;
+    const int b1 = bz / P.nb2, b2 = bz - b1 * P.nb2;
+    const zd* A = (const zd*)g.A + (long)b1 * dev_eval(g.sA1, d) + (long)b2 * dev_eval(g.sA2, d);
+    const zd* B = (const zd*)g.B + (long)b1 * dev_eval(g.sB1, d) + (long)b2 * dev_eval(g.sB2, d);
+    const int kbeg = kp * P.chunk, kend = min(P.K, kbeg + P.chunk);
+    // the products of padding rows are skipped where a whole warp would form only those
+    const int wrow = row0 + (TS == 16 ? 2 * ((tid >> 5) & 7) : 4 * ((tid >> 5) & 1));
+    const bool work = wrow < P.m;
+    cx<Cm> acc = mk<Cm>(GAcc<Cm>().value(), GAcc<Cm>().value());
+    for (int k0 = kbeg; k0 < kend; k0 += GB_K) {
+      zd v[2 * NL];  // all loads of a chunk in flight (three CTAs per SM cover their latency)
+#pragma unroll
+      for (int q = 0; q < NL; q++) {
+        const int e = tid + q * G_THREADS;
+        // op(A)(i, k): OP_N A[i lda + k]; OP_T, OP_C A[k lda + i] (lanes along the rows of memory)
+        const int kk = g.opA == OP_N ? e % GB_K : e / TS, i = g.opA == OP_N ? e / GB_K : e % TS;
+        const int gi = row0 + i, gk = k0 + kk;
+        v[q] = mk<double>(0.0, 0.0);
+        if (gi < P.m && gk < kend) v[q] = g.opA == OP_N ? A[(long)gi * lda + gk] : A[(long)gk * lda + gi];
+        // op(B)(k, j): OP_N B[k ldb + j]; OP_T, OP_C B[j ldb + k]
+        const int k2 = g.opB == OP_N ? e / TS : e % GB_K, j = g.opB == OP_N ? e % TS : e / GB_K;
+        const int gj = col0 + j, gl = k0 + k2;
+        v[NL + q] = mk<double>(0.0, 0.0);
+        if (gj < P.n && gl < kend) v[NL + q] = g.opB == OP_N ? B[(long)gl * ldb + gj] : B[(long)gj * ldb + gl];
+      }
+#pragma unroll
+      for (int q = 0; q < NL; q++) {
+        const int e = tid + q * G_THREADS;
+        const int kk = g.opA == OP_N ? e % GB_K : e / TS, i = g.opA == OP_N ? e / GB_K : e % TS;
+        if (g.opA == OP_C) v[q].im = -v[q].im;
+        As[kk * LD + i] = to_c((cx<Cm>*)nullptr, v[q]);
+        const int k2 = g.opB == OP_N ? e / TS : e % GB_K, j = g.opB == OP_N ? e % TS : e / GB_K;
+        if (g.opB == OP_C) v[NL + q].im = -v[NL + q].im;
+        Bs[k2 * LD + j] = to_c((cx<Cm>*)nullptr, v[NL + q]);
+      }
+      __syncthreads();
+      const int kn = min(GB_K, kend - k0);
+      // slice s takes the k of its residue modulo SL
+      auto step = [&](int kk, GAcc<Cm>& re, GAcc<Cm>& im) {
+        const cx<Cm> a = As[kk * LD + ty], b = Bs[kk * LD + tx];
+        re.mac(a.re, b.re);
+        re.mac(-a.im, b.im);
+        im.mac(a.re, b.im);
+        im.mac(a.im, b.re);
+        re.settle();
+        im.settle();
+      };
+      if (work) {
+        // even and odd steps apart and a sum of its own for every chunk: shorter chains, and
+        // less rounding (errors grow with the chain's length)
+        GAcc<Cm> re0, im0, re1, im1;
+        int kk = slice;
+#pragma unroll 2
+        for (; kk + SL < kn; kk += 2 * SL) {
+          step(kk, re0, im0);
+          step(kk + SL, re1, im1);
+        }
+        if (kk < kn) step(kk, re0, im0);
+        acc = mk<Cm>(acc.re + (re0.value() + re1.value()), acc.im + (im0.value() + im1.value()));
+      }
+      __syncthreads();
+    }
+    if (SL > 1) {
+      // the slices' sums, in slice order
+      As[slice * TS * TS + o] = acc;
+      __syncthreads();
+      if (slice == 0) {
+#pragma unroll
+        for (int q = 1; q < SL; q++) acc = cadd(acc, As[q * TS * TS + o]);
+      }
+      __syncthreads();
+    }
+    const bool mine = slice == 0 && row0 + ty < P.m && col0 + tx < P.n;
+    if (P.ks > 1) {
+      // partial tile of this K part; the last CTA of the tile adds them in order
+      if (mine) part_ws[((long)kp * P.ntiles + tile) * GB_TILE + o] = acc;
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) *s_last = atomicAdd(counters + tile, 1) == P.ks - 1;
+      __syncthreads();
+      const bool last = *s_last != 0;
+      __syncthreads();
+      if (!last) continue;
+      __threadfence();
+      if (mine) {
+        const long pstride = P.ntiles * GB_TILE;
+        const cx<Cm>* P0 = part_ws + tile * GB_TILE + o;
+        cx<Cm> sum = ldcg_cx(P0);
+        int q = 1;
+        // four independent loads in flight, added in part order
+        for (; q + 4 <= P.ks; q += 4) {
+          const cx<Cm> v0 = ldcg_cx(P0 + q * pstride), v1 = ldcg_cx(P0 + (q + 1) * pstride);
+          const cx<Cm> v2 = ldcg_cx(P0 + (q + 2) * pstride), v3 = ldcg_cx(P0 + (q + 3) * pstride);
+          sum = cadd(cadd(cadd(cadd(sum, v0), v1), v2), v3);
+        }
+        for (; q < P.ks; q++) sum = cadd(sum, ldcg_cx(P0 + q * pstride));
+        acc = sum;
+      }
+      if (tid == 0) counters[tile] = 0;  // ready for the next launch on this workspace
+    }
+    if (mine) {
+      const zd v = cmul(gemm_alpha(g), mk<double>((double)acc.re, (double)acc.im));
+      zd* dst = (zd*)g.C + (long)b1 * dev_eval(g.sC1, d) + (long)b2 * dev_eval(g.sC2, d) +
+                (long)(row0 + ty) * dev_eval(g.ldc, d) + col0 + tx;
+      *dst = g.beta ? cadd(v, *dst) : v;
+    }
+  }
+}
+
+// Cm: the type the products are formed and summed in (double, or double-float in the
+// mixed forms)
+template <typename Cm, bool GRP>
+__global__ void __launch_bounds__(G_THREADS, 3) k_gemm(const GemmDesc g_in, const int* __restrict__ d_in, double* prof,
+                                                       const GemmDesc* __restrict__ grp) {
   // grouped launch: this CTA works on member blockIdx.y, whose descriptor (and dims)
-  // come from the group's table (kept in shared memory, not registers); the K split
-  // is decided on the member's nominal grid
+  // come from the group's table (kept in shared memory, not registers); the tile and the K
+  // split are decided on the member's nominal grid
   __shared__ GemmDesc s_g;
+  __shared__ __align__(16) unsigned char sm[GB_SMEM * sizeof(cx<Cm>)];
+  __shared__ int s_last;
   if constexpr (GRP) {
-    if (threadIdx.x == 0) s_g = grp[blockIdx.y];
+    const int* src = (const int*)(grp + blockIdx.y);
+    for (int i = threadIdx.x; i < (int)(sizeof(GemmDesc) / sizeof(int)); i += G_THREADS) ((int*)&s_g)[i] = src[i];
     __syncthreads();
   }
   const GemmDesc& g = GRP ? s_g : g_in;
   const int* __restrict__ d = GRP ? s_g.dims : d_in;
   const int gnom = g.split_grid > 0 ? g.split_grid : (int)gridDim.x;
-  const int m = dev_eval(g.m, d), n = dev_eval(g.n, d), K = dev_eval(g.k, d);
-  const int nb1 = dev_eval(g.nb1, d), nb2 = dev_eval(g.nb2, d);
-  const int nb = nb1 * nb2;
-  if (m <= 0 || n <= 0 || nb <= 0) return;
-  const int tm = (m + GB_M - 1) / GB_M, tn = (n + GB_N - 1) / GB_N;
-  const long ntiles = (long)tm * tn * nb;
-  // the K split of this launch, from the run-time sizes (the same in every CTA)
-  int ks = 1;
-  if (g.ws && K > GB_K && ntiles < (long)gnom) {
+  GemmPlan P;
+  P.m = dev_eval(g.m, d);
+  P.n = dev_eval(g.n, d);
+  P.K = dev_eval(g.k, d);
+  P.nb1 = dev_eval(g.nb1, d);
+  P.nb2 = dev_eval(g.nb2, d);
+  const int nb = P.nb1 * P.nb2;
+  if (P.m <= 0 || P.n <= 0 || nb <= 0) return;
+  // the tile: both counts of tiles in waves over the SMs (a quarter of the nominal grid)
+  const long t16 = (long)((P.m + 15) / 16) * ((P.n + 15) / 16) * nb;
+  const long t8 = (long)((P.m + 7) / 8) * ((P.n + 7) / 8) * nb;
+  const int sms = max(1, gnom / 4);
+  const float c16 = (float)((t16 + sms - 1) / sms) * tile_cycles<Cm>(16, P.K);
+  const float c8 = (float)((t8 + sms - 1) / sms) * tile_cycles<Cm>(8, P.K);
+  const bool small = c8 < c16;
+  P.ntiles = small ? t8 : t16;
+  P.tm = small ? (P.m + 7) / 8 : (P.m + 15) / 16;
+  P.tn = small ? (P.n + 7) / 8 : (P.n + 15) / 16;
+  // the K split (the same in every CTA): parts of at least ~8,000 cycles, about twice what
+  // the partial tiles' round trip through L2 costs
+  P.ks = 1;
+  const int least = GB_K * (std::is_same<Cm, double>::value ? (small ? 2 : 1) : (small ? 8 : 2));
+  if (g.ws && P.K > least && P.ntiles < (long)gnom) {
     const int cap = g.ksplit >= 1 ? g.ksplit : GB_SPLIT_CAP;
-    ks = (int)min((long)cap, (long)gnom / ntiles);
-    ks = min(ks, (K + GB_K - 1) / GB_K);
-    if (ks < 1) ks = 1;
+    P.ks = (int)min((long)cap, (long)gnom / P.ntiles);
+    P.ks = max(1, min(P.ks, (P.K + least - 1) / least));
   }
-  const int chunk = ks > 1 ? (((K + ks - 1) / ks + GB_K - 1) / GB_K) * GB_K : K;
-  if (ks > 1) ks = (K + chunk - 1) / chunk;
+  P.chunk = P.ks > 1 ? (((P.K + P.ks - 1) / P.ks + GB_K - 1) / GB_K) * GB_K : P.K;
+  if (P.ks > 1) P.ks = (P.K + P.chunk - 1) / P.chunk;
   if (prof && blockIdx.x == 0 && threadIdx.x == 0) {
-    atomicAdd(prof, 8.0 * (double)m * (double)n * (double)K * nb);
-    atomicAdd(prof + QLB_K_COUNT, (double)sizeof(cx<R>) * ((double)m * K + (double)K * n + (double)m * n) * nb);
+    atomicAdd(prof, 8.0 * (double)P.m * (double)P.n * (double)P.K * nb);
+    atomicAdd(prof + QLB_K_COUNT,
+              (double)sizeof(zd) * ((double)P.m * P.K + (double)P.K * P.n + (double)P.m * P.n) * nb);
   }
-  const long lda = dev_eval(g.lda, d), ldb = dev_eval(g.ldb, d), ldc = dev_eval(g.ldc, d);
-  cx<Cm>* part_ws = (cx<Cm>*)g.ws;
-  int* counters = g.ws ? (int*)(part_ws + (long)gnom * GB_TILE) : nullptr;
-
-  __shared__ cx<Cm> As[GB_K][GB_M + 1];
-  __shared__ cx<Cm> Bs[GB_K][GB_N + 1];
-  __shared__ int s_last;
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const long items = ntiles * ks;
-  for (long it = blockIdx.x; it < items; it += gridDim.x) {
-    const long tile = it / ks;
-    const int kp = (int)(it - tile * ks);
-    const int bz = (int)(tile / ((long)tm * tn));
-    const int t2 = (int)(tile - (long)bz * tm * tn);
-    const int row0 = (t2 / tn) * GB_M, col0 = (t2 % tn) * GB_N;
-    const int b1 = bz / nb2, b2 = bz - b1 * nb2;
-    const cx<R>* A = (const cx<R>*)g.A + (long)b1 * dev_eval(g.sA1, d) + (long)b2 * dev_eval(g.sA2, d);
-    const cx<R>* B = (const cx<R>*)g.B + (long)b1 * dev_eval(g.sB1, d) + (long)b2 * dev_eval(g.sB2, d);
-    cx<R>* C = (cx<R>*)g.C + (long)b1 * dev_eval(g.sC1, d) + (long)b2 * dev_eval(g.sC2, d);
-    const int kbeg = kp * chunk, kend = min(K, kbeg + chunk);
-
-    // warp-uniform: does this warp own an output row of the tile (rows 2w, 2w + 1
-    // of each half), and does the tile reach the upper column half
-    const int wrow = row0 + 2 * (tid >> 5);
-    const bool do_r0 = wrow < m, do_r1 = wrow + 16 < m, do_c1 = col0 + 16 < n;
-    cx<Cm> acc[2][2];
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-      for (int j = 0; j < 2; j++) acc[i][j] = to_c<Cm>(mk<R>(0, 0));
-    for (int k0 = kbeg; k0 < kend; k0 += GB_K) {
-      // A tile: rows row0.., cols k0..
-      for (int e = tid; e < GB_M * GB_K; e += G_THREADS) {
-        int i, kk;
-        if (g.opA == OP_N) {
-          kk = e % GB_K;
-          i = e / GB_K;
-        } else {
-          i = e % GB_M;
-          kk = e / GB_M;
-        }
-        int gi = row0 + i, gk = k0 + kk;
-        As[kk][i] = to_c<Cm>((gi < m && gk < kend) ? ldop(A, g.opA, lda, gi, gk) : mk<R>(0, 0));
-      }
-      for (int e = tid; e < GB_N * GB_K; e += G_THREADS) {
-        int j, kk;
-        if (g.opB == OP_N) {
-          j = e % GB_N;
-          kk = e / GB_N;
-        } else {
-          kk = e % GB_K;
-          j = e / GB_K;
-        }
-        int gj = col0 + j, gk = k0 + kk;
-        // op(B)(k, j): OP_N B[k*ldb + j]; OP_T B[j*ldb + k]
-        cx<R> v = mk<R>(0, 0);
-        if (gj < n && gk < kend) {
-          if (g.opB == OP_N)
-            v = B[(long)gk * ldb + gj];
-          else {
-            v = B[(long)gj * ldb + gk];
-            if (g.opB == OP_C) v.im = -v.im;
-          }
-        }
-        Bs[kk][j] = to_c<Cm>(v);
-      }
-      __syncthreads();
-      // the products of the padding are skipped where a whole warp would form only
-      // padding (warp-uniform tests: the warp's rows, the upper column half, the
-      // K tail), which on the slow FP64 pipe is most of the work of a small GEMM
-      const int kn = min(GB_K, kend - k0);
-      if (kn == GB_K && do_r1 && do_c1) {
-#pragma unroll
-        for (int kk = 0; kk < GB_K; kk++) {
-          cx<Cm> a0 = As[kk][ty], a1 = As[kk][ty + 16];
-          cx<Cm> b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-          cmac(acc[0][0], a0, b0);
-          cmac(acc[0][1], a0, b1);
-          cmac(acc[1][0], a1, b0);
-          cmac(acc[1][1], a1, b1);
-        }
-      } else if (do_r0) {
-#pragma unroll 4
-        for (int kk = 0; kk < kn; kk++) {
-          cx<Cm> a0 = As[kk][ty];
-          cx<Cm> b0 = Bs[kk][tx];
-          cmac(acc[0][0], a0, b0);
-          if (do_c1) cmac(acc[0][1], a0, Bs[kk][tx + 16]);
-          if (do_r1) {
-            cx<Cm> a1 = As[kk][ty + 16];
-            cmac(acc[1][0], a1, b0);
-            if (do_c1) cmac(acc[1][1], a1, Bs[kk][tx + 16]);
-          }
-        }
-      }
-      __syncthreads();
-    }
-    if (ks > 1) {
-      // partial tile of this K part; the last CTA of the tile adds them in order
-      cx<Cm>* P = part_ws + ((long)kp * ntiles + tile) * GB_TILE;
-      // (only the entries inside the output are written and read back)
-#pragma unroll
-      for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 2; j++)
-          if (row0 + ty + 16 * i < m && col0 + tx + 16 * j < n) P[(ty + 16 * i) * GB_N + tx + 16 * j] = acc[i][j];
-      __threadfence();
-      __syncthreads();
-      if (tid == 0) s_last = atomicAdd(counters + tile, 1) == ks - 1;
-      __syncthreads();
-      if (!s_last) continue;
-      __threadfence();
-#pragma unroll
-      for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 2; j++) {
-          if (row0 + ty + 16 * i >= m || col0 + tx + 16 * j >= n) continue;
-          cx<Cm> sum = to_c<Cm>(mk<R>(0, 0));
-          const long off = (long)(ty + 16 * i) * GB_N + tx + 16 * j;
-          const long pstride = ntiles * GB_TILE;
-          const cx<Cm>* P0 = part_ws + tile * GB_TILE + off;
-          int s = 0;
-          // four independent loads in flight, added in part order
-          for (; s + 4 <= ks; s += 4) {
-            const cx<Cm> v0 = ldcg_cx(P0 + s * pstride), v1 = ldcg_cx(P0 + (s + 1) * pstride);
-            const cx<Cm> v2 = ldcg_cx(P0 + (s + 2) * pstride), v3 = ldcg_cx(P0 + (s + 3) * pstride);
-            sum = cadd(cadd(cadd(cadd(sum, v0), v1), v2), v3);
-          }
-          for (; s < ks; s++) sum = cadd(sum, ldcg_cx(P0 + s * pstride));
-          acc[i][j] = sum;
-        }
-      if (tid == 0) counters[tile] = 0;  // ready for the next launch on this workspace
-    }
-    const cx<R> alpha = gemm_alpha<R>(g);
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-      for (int j = 0; j < 2; j++) {
-        int gi = row0 + ty + 16 * i, gj = col0 + tx + 16 * j;
-        if (gi < m && gj < n) {
-          cx<R> v = cmul(alpha, to_s<R>(acc[i][j]));
-          cx<R>* dst = C + (long)gi * ldc + gj;
-          if (g.beta) v = cadd(v, *dst);
-          *dst = v;
-        }
-      }
-  }
+  if ((long)blockIdx.x >= P.ntiles * P.ks) return;
+  if (small)
+    gemm_items<Cm, 8>(g, d, P, gnom, sm, &s_last);
+  else
+    gemm_items<Cm, 16>(g, d, P, gnom, sm, &s_last);
 }
 
 }  // namespace
@@ -279,49 +332,42 @@ int gemm_grid_default() {
       cudaGetLastError();
       sms = 148;
     }
-    grid = 2 * sms;
+    grid = 4 * sms;
   }
   return grid;
 }
 
-template <typename R>
 cudaError_t launch_gemm(const GemmDesc& g, const int* d_dims, cudaStream_t s, double* prof) {
-  const long planned = (long)((g.m_max + GB_M - 1) / GB_M) * ((g.n_max + GB_N - 1) / GB_N) *
-                       (g.nb_max > 0 ? g.nb_max : 1);
+  const long planned =
+      (long)((g.m_max + 7) / 8) * ((g.n_max + 7) / 8) * (g.nb_max > 0 ? g.nb_max : 1);
   if (planned <= 0) return cudaSuccess;
-  // with a workspace: a fixed grid that the run-time split fills; without: one CTA
-  // per planned tile (persistent above 4096)
-  const int grid = g.ws ? (g.grid > 0 ? g.grid : gemm_grid_default()) : (int)std::min<long>(planned, 4096);
+  // a fixed grid that the run-time decomposition fills; without a workspace (no K split)
+  // no more CTAs than planned tiles
   GemmDesc gg = g;
-  if (!g.ws) gg.ksplit = 1;
-  gg.split_grid = 0;
-  if constexpr (std::is_same<R, double>::value) {
-    if (g.df64) {
-      k_gemm<R, df64, false><<<grid, G_THREADS, 0, s>>>(gg, d_dims, prof, nullptr);
-      return cudaGetLastError();
-    }
-  }
-  k_gemm<R, R, false><<<grid, G_THREADS, 0, s>>>(gg, d_dims, prof, nullptr);
+  const int full = g.ws && g.grid > 0 ? g.grid : gemm_grid_default();
+  const int grid = g.ws ? full : (int)std::min<long>(planned, full);
+  gg.split_grid = full;
+  if (g.df64)
+    k_gemm<df64, false><<<grid, G_THREADS, 0, s>>>(gg, d_dims, prof, nullptr);
+  else
+    k_gemm<double, false><<<grid, G_THREADS, 0, s>>>(gg, d_dims, prof, nullptr);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_gemm<double>(const GemmDesc&, const int*, cudaStream_t, double*);
-template cudaError_t launch_gemm<float>(const GemmDesc&, const int*, cudaStream_t, double*);
-
 // The same GEMM of S states in one launch: grid (per-member CTAs, S).  Every member
 // descriptor in d_grp carries its dims, a workspace for the default grid and
-// split_grid = the default grid, so each member is split and summed exactly as in
+// split_grid = the default grid, so each member is tiled, split and summed exactly as in
 // its own launch; the per-member CTA count only changes how the work items are
-// shared out (S x per-member CTAs ~ two per SM over the whole group).
+// shared out (S x per-member CTAs ~ four per SM over the whole group).
 cudaError_t launch_gemm_group(const GemmDesc* d_grp, int S, int use_df, cudaStream_t s, double* prof) {
   if (S <= 0) return cudaSuccess;
   const int full = gemm_grid_default();
   const int per = std::max(8, std::min(full, (full + S - 1) / S));
   GemmDesc dummy{};
   if (use_df)
-    k_gemm<double, df64, true><<<dim3(per, S), G_THREADS, 0, s>>>(dummy, nullptr, prof, d_grp);
+    k_gemm<df64, true><<<dim3(per, S), G_THREADS, 0, s>>>(dummy, nullptr, prof, d_grp);
   else
-    k_gemm<double, double, true><<<dim3(per, S), G_THREADS, 0, s>>>(dummy, nullptr, prof, d_grp);
+    k_gemm<double, true><<<dim3(per, S), G_THREADS, 0, s>>>(dummy, nullptr, prof, d_grp);
   return cudaGetLastError();
 }
 

@@ -114,7 +114,7 @@ struct GemmDesc {
   int kclass;  // profiling class
   // Work distribution.  Without ws: one CTA per planned output tile.  With ws (at
   // least gemm_workspace_elems(grid) complex elements, zeroed once): a fixed grid of
-  // `grid` CTAs (0 = two per SM) that splits the K range at run time so that tiles x
+  // `grid` CTAs (0 = four per SM) that splits the K range at run time so that tiles x
   // parts fill it; ksplit >= 1 caps that split (0: the default cap).  The last CTA of a tile adds the
   // partials in part order (deterministic).
   int ksplit;

@@ -245,7 +245,7 @@ static qlb_status gemm(qlb_state* st, GemmDesc& g) {
   // 3xTF32 on tcgen05; everything feeding a truncation decision stays FP64
   cudaError_t e = (st->prec == QLB_PREC_TC && g.kclass == QLB_K_CONTRACT)
                       ? launch_gemm_tc(g, st->d_dims, st->stream, st->d_err, pf)
-                      : launch_gemm<double>(g, st->d_dims, st->stream, pf);
+                      : launch_gemm(g, st->d_dims, st->stream, pf);
   prof_after(ctx, st->stream, g.kclass, a);
   if (e != cudaSuccess) {
     set_error(std::string("gemm launch: ") + cudaGetErrorString(e));
@@ -1213,7 +1213,7 @@ qlb_status expectation_mpo(qlb_state* st, const std::vector<zd*>& W, const std::
     g.m_max = Dl;
     g.n_max = 2 * (int)cap(i + 1);
     g.nb_max = (int)cap(i);
-    QLB_CUDA_TRY(launch_gemm<double>(g, st->d_dims, st->stream, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, st->d_dims, st->stream, nullptr));
     g = gdesc();
     g.A = Y;
     g.B = W[i];
@@ -1234,7 +1234,7 @@ qlb_status expectation_mpo(qlb_state* st, const std::vector<zd*>& W, const std::
     g.m_max = (int)cap(i + 1);
     g.n_max = Dr;
     g.nb_max = 2 * (int)cap(i);
-    QLB_CUDA_TRY(launch_gemm<double>(g, st->d_dims, st->stream, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, st->d_dims, st->stream, nullptr));
     g = gdesc();
     g.A = st->site[i];
     g.B = Z;
@@ -1248,7 +1248,7 @@ qlb_status expectation_mpo(qlb_state* st, const std::vector<zd*>& W, const std::
     g.ldc = dvar(SB(i + 1), Dr);
     g.m_max = (int)cap(i + 1);
     g.n_max = (int)cap(i + 1) * Dr;
-    QLB_CUDA_TRY(launch_gemm<double>(g, st->d_dims, st->stream, nullptr));
+    QLB_CUDA_TRY(launch_gemm(g, st->d_dims, st->stream, nullptr));
     std::swap(E0, E1);
   }
   zd res;

@@ -105,7 +105,7 @@ QLB_API qlb_status qlb_autotune(qlb_ctx* ctx, const char* path) {
         float t = 1e30f;
         for (int rep = 0; rep < 4; rep++) {
           cudaEventRecord(a, 0);
-          cudaError_t e = launch_gemm<double>(g, nullptr, 0, nullptr);
+          cudaError_t e = launch_gemm(g, nullptr, 0, nullptr);
           cudaEventRecord(b, 0);
           if (e == cudaSuccess) e = cudaEventSynchronize(b);
           if (e != cudaSuccess) {
