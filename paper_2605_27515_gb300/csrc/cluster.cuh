@@ -13,8 +13,13 @@ namespace qlb {
 
 namespace {
 
-constexpr int FC_NT = 256;  // threads per CTA
-constexpr int FC_NW = FC_NT / 32;
+// Threads per CTA: FP64 one warp for each of the SM's four partitions, as a warp-wide FP64
+// instruction holds a partition's pipe for 64 clocks and what every warp computes for itself
+// (norms, thresholds, candidates) is paid per warp; double-float two, to cover its chains.
+template <typename R>
+struct ClThreads {
+  static constexpr int v = std::is_same<R, double>::value ? 128 : 256;
+};
 constexpr int FC_MAX_N = 256;
 constexpr int FC_MAX_C = 16;
 // Residuals under 1e-30 of the trace (amplitudes 1e-15 of the state's) are not taken as
@@ -123,6 +128,12 @@ template <typename R>
 __device__ __forceinline__ cx<R> csub_r(cx<R> a, cx<R> b) {
   return mk<R>(a.re - b.re, a.im - b.im);
 }
+
+// a <= b for finite a and b >= 0 (doubles: by their bit patterns, off the FP64 pipe)
+__device__ __forceinline__ bool le_nn(double a, double b) {
+  return __double_as_longlong(a) <= __double_as_longlong(b);
+}
+__device__ __forceinline__ bool le_nn(df64 a, df64 b) { return a <= b; }
 
 // 1 / sqrt(w) for w in FP32's normal range: FP32 seed y (relative error e / 2 ~ 1e-7)
 // and one third-order step, y (1 + e/2 + 3 e^2 / 8) with e = 1 - w y^2, so no division

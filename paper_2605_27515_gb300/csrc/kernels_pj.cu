@@ -36,9 +36,9 @@
 // bits, whatever larger size it was launched for; CTAs beyond C leave at once.
 //
 // Measured on GB300, cold Gram matrices of rank n with weights over 1e-12 (against the
-// two-sided Jacobi solves of kernels_eig.cu): FP64 n = 16 194 us (698), n = 32 460 us
-// (1,925), n = 64 1.31 ms (6.03), n = 128 4.21 ms (38.8); double-float n = 16 102 us (388),
-// n = 32 266 us (1,251), n = 64 0.69 ms (3.83), n = 128 2.05 ms (23.8).  At n = 64 an FP64 round of
+// two-sided Jacobi solves of kernels_eig.cu): FP64 n = 16 188 us (698), n = 32 446 us
+// (1,925), n = 64 1.28 ms (6.03), n = 128 4.14 ms (38.8); double-float n = 16 100 us (388),
+// n = 32 264 us (1,251), n = 64 0.69 ms (3.83), n = 128 2.05 ms (23.8).  At n = 64 an FP64 round of
 // four pairs to a CTA takes 4,700 cycles, ~3,500 of them the FP64 pipe; a double-float
 // round 2,100, the latency of its chain.
 //
@@ -52,8 +52,7 @@ namespace qlb {
 
 namespace {
 
-constexpr int PJ_NT = FC_NT;
-constexpr int PJ_NW = FC_NW;
+constexpr int PJ_MAX_NW = 8;  // warps per CTA at most
 constexpr int PJ_MAX_N = FC_MAX_N;
 constexpr int PJ_MAX_C = FC_MAX_C;
 constexpr int PJ_SLOTS = PJ_MAX_N + 2 * PJ_MAX_C;  // columns with the padding of the last block
@@ -84,7 +83,7 @@ struct __align__(16) FactorSmem {
   unsigned char d[FC_MAX_N * 8];     // residual diagonal of our rows
   unsigned char floor[FC_MAX_N * 8]; // below it only rounding is left
   unsigned char open[FC_MAX_N];      // our rows not taken as pivots yet
-  double red[FC_NW];
+  double red[PJ_MAX_NW];
   unsigned long long cbar;           // every working CTA has arrived
   unsigned key[3];                   // our best pivot candidate
   int bad;
@@ -122,6 +121,7 @@ __device__ __forceinline__ bool factor_begin(FactorSmem& fs, unsigned long long*
 template <typename R>
 __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd* G, int n, int ca, int rank,
                                    cx<R>* Gl, cx<R>* Ll) {
+  constexpr int NT = ClThreads<R>::v, NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const R zero = pzero(R());
   cx<R>* const s_row = (cx<R>*)fs.row;
@@ -142,12 +142,12 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
 
   // trace, scale, our rows
   double tr = 0.0;
-  for (int i = tid; i < n; i += FC_NT) tr += ::fabs(G[(long)i * n + i].re);
+  for (int i = tid; i < n; i += NT) tr += ::fabs(G[(long)i * n + i].re);
   for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
   if (lane == 0) fs.red[warp] = tr;
   __syncthreads();
   tr = fs.red[0];
-  for (int w = 1; w < FC_NW; w++) tr += fs.red[w];
+  for (int w = 1; w < NW; w++) tr += fs.red[w];
   const bool tr_ok = ::isfinite(tr) && tr > 0.0;
   const int ex = tr_ok ? max(-1000, min(1000, ilogb(tr))) : 0;
   const double up = ldexp(1.0, -ex);
@@ -155,7 +155,7 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
   out.down = ldexp(1.0, ex);
   const R eps = R(FcEps<R>::pivot);
   bool bad = !::isfinite(tr);
-  for (int x = tid; x < nl * n; x += FC_NT) {
+  for (int x = tid; x < nl * n; x += NT) {
     const int li = x / n, j = x - li * n;
     const zd v = G[(long)r0 * n + x];
     bad = bad || !::isfinite(v.re) || !::isfinite(v.im);
@@ -175,7 +175,7 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
   const int want = std::is_same<R, double>::value ? 4 : 8;
   int LR = 32;
   while (LR > 4 && (rpb * LR + 31) / 32 > want) LR >>= 1;
-  const int rg = tid / LR, rl = tid % LR, nrg = FC_NT / LR;
+  const int rg = tid / LR, rl = tid % LR, nrg = NT / LR;
   // a candidate pivot: FP32 bits of its residual with the low byte replaced by the
   // index's complement (the pivot is the largest to 2^-15, ties to the lower row)
   auto key_of = [&](int li) -> unsigned {
@@ -186,7 +186,7 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
   };
   {
     unsigned key = 0;
-    for (int li = tid; li < nl; li += FC_NT) key = max(key, key_of(li));
+    for (int li = tid; li < nl; li += NT) key = max(key, key_of(li));
     key = __reduce_max_sync(0xffffffffu, key);
     if (lane == 0 && key) atomicMax(&fs.key[0], key);
   }
@@ -208,14 +208,14 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
       const R dp = *on_cta(&s_d[lp], op);  // stays as it is while its row is the pivot's
       if (ca > 1) {
         const cx<R>* rem = on_cta(row, op);
-        for (int t = tid; t < r; t += FC_NT) s_row[t] = rem[t];
+        for (int t = tid; t < r; t += NT) s_row[t] = rem[t];
         row = s_row;
         __syncthreads();
       }
-      const R inv = rsqrt_r(dp);
       unsigned best = 0;
       for (int i0 = 0; i0 < nl; i0 += nrg) {
         if (i0 + (warp * 32) / LR >= nl) break;  // no row for this warp
+        const R inv = rsqrt_r(dp);
         const int li = i0 + rg;
         const bool act = li < nl;
         Acc<R> cr, ci;
@@ -267,8 +267,9 @@ struct __align__(16) PjSweep {
 // ------------------------------------------------------------------ the kernel
 
 template <typename R, bool GRP>
-__global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d, double* prof,
+__global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* __restrict__ d, double* prof,
                                              const EigDesc* __restrict__ grp) {
+  constexpr int NT = ClThreads<R>::v, NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (GRP) {  // grouped launch: one cluster per member (blockIdx.y; the cluster spans x)
     e = grp[blockIdx.y];
@@ -290,8 +291,8 @@ __global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d,
   __shared__ FactorSmem fs;
   // read by the other CTAs after a barrier; two sets in turn, as a set is written again
   // only after the barrier that follows their reads
-  __shared__ PjSweep s_sweep[2][PJ_NW];
-  __shared__ double s_off[PJ_NW];
+  __shared__ PjSweep s_sweep[2][NW];
+  __shared__ double s_off[NW];
   __shared__ double s_own[PJ_MAX_N + 2];  // squared norms of our columns
   __shared__ double s_lam[PJ_SLOTS], s_w[PJ_SLOTS];
   __shared__ short s_rank[PJ_SLOTS];
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d,
   const int ld = n + 1;  // a column and its squared norm
   cx<R>* cur = buf0;
   cx<R>* nxt = buf1;
-  for (int x = tid; x < nc * n; x += PJ_NT) {
+  for (int x = tid; x < nc * n; x += NT) {
     const int i = x / nc, s = x - i * nc;
     const int t = s < b ? rank * b + s : (ca + rank) * b + (s - b);
     const int o = i / rpb;
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d,
   const int want = std::is_same<R, double>::value ? 4 : 8;
   int LP = 32;
   while (LP > 4 && ((b * LP + 31) / 32 > want || LP >= 2 * n)) LP >>= 1;
-  const int pg = tid / LP, pl = tid % LP, npg = PJ_NT / LP;
+  const int pg = tid / LP, pl = tid % LP, npg = NT / LP;
   const unsigned gmask = (LP == 32 ? 0xffffffffu : ((1u << LP) - 1u) << (lane & ~(LP - 1)));
   const float tol_f = (float)(FcEps<R>::v * (double)(n > 8 ? n : 8));
   auto norm2 = [&](int k) {  // squared norm of column k, in every lane of its group
@@ -488,13 +489,13 @@ __global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d,
       for (int s = 16; s > 0; s >>= 1) off_l += __shfl_xor_sync(0xffffffffu, off_l, s);
       if (lane == 0) s_off[warp] = off_l;
       csync();
-      for (int c = 0; c < ca * PJ_NW; c++) off2 += *on_cta(&s_off[c % PJ_NW], c / PJ_NW);
+      for (int c = 0; c < ca * NW; c++) off2 += *on_cta(&s_off[c % NW], c / NW);
       break;
     }
     int all = 0;
     float amc = 0.f, ams = 0.f;
-    for (int c = lane; c < ca * PJ_NW; c += 32) {
-      const PjSweep v = *on_cta(&s_sweep[sweep & 1][c % PJ_NW], c / PJ_NW);
+    for (int c = lane; c < ca * NW; c += 32) {
+      const PjSweep v = *on_cta(&s_sweep[sweep & 1][c % NW], c / NW);
       all += v.nrot;
       amc = fmaxf(amc, v.mc);
       ams = fmaxf(ams, v.ms);
@@ -526,11 +527,11 @@ __global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d,
     if (k < nc && pl == 0) s_own[k] = (double)na * down;
   }
   csync();
-  for (int i = tid; i < ns; i += PJ_NT) s_lam[i] = *on_cta(&s_own[i % nc], i / nc);
+  for (int i = tid; i < ns; i += NT) s_lam[i] = *on_cta(&s_own[i % nc], i / nc);
   csync();  // the last access to another CTA's shared memory
   if (tid == 0) s_bad = any_bad ? 1 : 0;
   __syncthreads();
-  for (int i = tid; i < ns; i += PJ_NT) {
+  for (int i = tid; i < ns; i += NT) {
     // squared norms order like their bit patterns
     const long long li = __double_as_longlong(s_lam[i]);
     if (!::isfinite(s_lam[i])) s_bad = 1;
@@ -616,15 +617,15 @@ __global__ void __launch_bounds__(PJ_NT, 1) k_pj(EigDesc e, int* __restrict__ d,
   __syncthreads();
   const int k = s_k;
   if (rank == 0 && e.lam)
-    for (int i = tid; i < n; i += PJ_NT) e.lam[i] = r > 0 && i < ns ? s_w[i] : 0.0;
+    for (int i = tid; i < n; i += NT) e.lam[i] = r > 0 && i < ns ? s_w[i] : 0.0;
   zd* out = (zd*)e.out;
   if (e.out_mode != 0 && e.out_mode != 1) return;
   if (r == 0) {  // nothing above rounding (or non-finite entries): one unit vector
     if (rank == 0)
-      for (int i = tid; i < n; i += PJ_NT) out[i] = mk<double>(i == 0 ? 1.0 : 0.0, 0.0);
+      for (int i = tid; i < n; i += NT) out[i] = mk<double>(i == 0 ? 1.0 : 0.0, 0.0);
     return;
   }
-  for (int s = warp; s < nc; s += PJ_NW) {
+  for (int s = warp; s < nc; s += NW) {
     const int rk = s_rank[rank * nc + s];
     if (rk >= k) continue;
     // the norm again in the working precision (a scaled weight may have left its range)
@@ -664,7 +665,7 @@ cudaError_t launch_pj(int n_max, const EigDesc& e, const int* d_dims, cudaStream
   cudaLaunchConfig_t cfg = {};
   const int c = pj_ctas<R>(n_max);
   cfg.gridDim = dim3(c, S, 1);
-  cfg.blockDim = dim3(PJ_NT, 1, 1);
+  cfg.blockDim = dim3(ClThreads<R>::v, 1, 1);
   cfg.dynamicSmemBytes = pj_smem<R>(n_max);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

@@ -32,8 +32,10 @@
 //
 // Measured on GB300, a cold G of rank r with weights over 1e-12 (against one CTA of 512
 // threads sweeping all columns, the kernel of the sizes above 256): FP64 n = 32, r = 16
-// 174 us (360), n = 64, r = 32 333 us (987), n = 128, r = 64 0.94 ms (4.47); double-float
-// 81 us (124), 280 us (348), 0.73 ms (2.25).
+// 143 us (360), n = 64, r = 32 274 us (987), n = 128, r = 64 0.84 ms (4.47); double-float
+// 79 us (124), 270 us (348), 0.71 ms (2.25).  FP64 on four warps instead of eight, with its
+// comparisons off the FP64 pipe, is 31 us, 59 us and 0.10 ms of that: what every warp
+// computes for itself held the pipes for ~6,000 of a step's ~20,000 cycles.
 //
 // R = double (the FP64 form) or df64 (the mixed forms).  G and U are FP64 in both.
 
@@ -77,8 +79,9 @@ struct __align__(16) Candidate {
 };
 
 template <typename R, bool GRP>
-__global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__ d, double* prof,
+__global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* __restrict__ d, double* prof,
                                                  const EigDesc* __restrict__ grp) {
+  constexpr int NT = ClThreads<R>::v, NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (GRP) {  // grouped launch: one cluster per member (blockIdx.y; the cluster spans x)
     e = grp[blockIdx.y];
@@ -104,9 +107,9 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
   __shared__ __align__(16) unsigned char y_raw[FC_MAX_N * sizeof(cx<R>)];
   __shared__ __align__(16) unsigned char z_raw[32 * sizeof(cx<R>)];
   __shared__ __align__(16) unsigned char c_raw[RB_LOCAL * sizeof(cx<R>)];
-  __shared__ __align__(16) unsigned char part_raw[FC_NW * sizeof(Cand)];
+  __shared__ __align__(16) unsigned char part_raw[NW * sizeof(Cand)];
   __shared__ __align__(16) unsigned char pub_raw[2 * sizeof(Cand)];
-  __shared__ __align__(16) unsigned char red_raw[FC_NW * 2 * sizeof(R)];
+  __shared__ __align__(16) unsigned char red_raw[NW * 2 * sizeof(R)];
   __shared__ __align__(16) unsigned char sums_raw[2 * sizeof(R)];
   cx<R>* const s_v = (cx<R>*)v_raw;      // the pivot column, then the new basis vector (a copy in every CTA)
   cx<R>* const s_y = (cx<R>*)y_raw;      // our basis vectors' part of Q Q^dag v; read by the others
@@ -150,17 +153,17 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
   // power-of-two scale from the trace, then W = G column by column: column k of a Hermitian
   // G is the conjugate of row k
   double trd = 0.0;
-  for (int i = tid; i < n; i += FC_NT) trd += ::fabs(G[(long)i * n + i].re);
+  for (int i = tid; i < n; i += NT) trd += ::fabs(G[(long)i * n + i].re);
   for (int o = 16; o > 0; o >>= 1) trd += __shfl_xor_sync(0xffffffffu, trd, o);
   if (lane == 0) ((double*)red_raw)[warp] = trd;
   __syncthreads();
   trd = ((double*)red_raw)[0];
-  for (int w = 1; w < FC_NW; w++) trd += ((double*)red_raw)[w];
+  for (int w = 1; w < NW; w++) trd += ((double*)red_raw)[w];
   const int ex = ::isfinite(trd) && trd > 0.0 ? max(-1000, min(1000, ilogb(trd))) : 0;
   const double up = ldexp(1.0, -ex);
   bool bad = !::isfinite(trd);
   Acc<R> fr_a, tr_a;
-  for (int x = tid; x < ncl * n; x += FC_NT) {
+  for (int x = tid; x < ncl * n; x += NT) {
     const int lk = x / n, i = x - lk * n;
     const zd g = G[(long)k0c * n + x];
     bad = bad || !::isfinite(g.re) || !::isfinite(g.im);
@@ -170,20 +173,18 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
     fr_a.mac(w.im, w.im);
     if (i == k0c + lk) tr_a.mac(w.re, from_f(R(), 1.f));
   }
-  for (int i = tid; i < RB_LOCAL; i += FC_NT) s_done[i] = 0;
+  for (int i = tid; i < RB_LOCAL; i += NT) s_done[i] = 0;
   if (bad) s_bad = 1;
   __syncthreads();
-  // sum of two values over the CTA, the same in every thread
+  // sums of two values over the CTA, the same in every thread
   auto cta_sum2 = [&](Acc<R> a, Acc<R> b, R& sa, R& sb) {
     const R h = csum(a, b, 32);
     if (lane < 2) s_red[2 * warp + lane] = h;
     __syncthreads();
-    sa = s_red[0];
-    sb = s_red[1];
-    for (int w = 1; w < FC_NW; w++) {
-      sa = sa + s_red[2 * w];
-      sb = sb + s_red[2 * w + 1];
-    }
+    R v = s_red[lane & (2 * NW - 1)];
+    for (int o = 2; o < 2 * NW; o <<= 1) v = v + sx(v, o);
+    sa = sget(v, 0);
+    sb = sget(v, 1);
     __syncthreads();
   };
   R fr, tr;
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
   const int want = std::is_same<R, double>::value ? 4 : 8;
   int LG = 32;
   while (LG > 4 && ((cpb * LG + 31) / 32 > want || LG >= 2 * n)) LG >>= 1;
-  const int g = tid / LG, gl = tid % LG, ng = FC_NT / LG;
+  const int g = tid / LG, gl = tid % LG, ng = NT / LG;
   const int base = lane & ~(LG - 1);
   // One sweep over our open columns: w_k -= q (q^dag w_k) if q; then the candidate with the
   // largest squared residual norm (ties to the lower column) and the residual weight.
@@ -221,7 +222,8 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
         a.re = sget(h, base);
         a.im = sget(h, base | 1);
       }
-      Acc<R> nu, dk;
+      Acc<R> nu, none;
+      R dk = zero;
       if (act)
         for (int i = gl; i < n; i += LG) {
           cx<R> w = wk[i];
@@ -233,10 +235,10 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
           }
           nu.mac(w.re, w.re);
           nu.mac(w.im, w.im);
-          if (i == k0c + k) dk.mac(w.re, from_f(R(), 1.f));
+          if (i == k0c + k) dk = w.re;
         }
-      const R h = csum(nu, dk, LG);
-      const R nuv = sget(h, base), dkv = sget(h, base | 1);
+      const R nuv = sget(csum(nu, none, LG), base);
+      const R dkv = sget(dk, base | ((k0c + k) & (LG - 1)));  // the lane of row k
       if (act && gl == 0) {
         const unsigned h2 = __float_as_uint(to_f(nuv)), l2 = 0xffffffffu - (unsigned)(k0c + k);
         if (lo == 0 || h2 > hi || (h2 == hi && l2 > lo)) {
@@ -263,12 +265,12 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
     if (ca > 1) {
       __syncthreads();
       if (warp == 0) {
-        const Cand c = s_part[lane & (FC_NW - 1)];
+        const Cand c = s_part[lane & (NW - 1)];
         const unsigned h = __reduce_max_sync(0xffffffffu, c.hi);
         const unsigned l = __reduce_max_sync(0xffffffffu, c.hi == h ? c.lo : 0u);
         const unsigned w = __ballot_sync(0xffffffffu, c.hi == h && c.lo == l);
         R ws = c.weight;
-        for (int o = 1; o < FC_NW; o <<= 1) ws = ws + sx(ws, o);
+        for (int o = 1; o < NW; o <<= 1) ws = ws + sx(ws, o);
         const R bv = sget(c.best, __ffs(w) - 1);
         if (lane == 0) {
           Cand p;
@@ -311,9 +313,9 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
     for (int par = 0;; j++, par ^= 1) {
       // the candidates, reduced alike in every warp of every CTA
       Cand c;
-      const int ne = ca == 1 ? FC_NW : ca;
+      const int ne = ca == 1 ? NW : ca;
       if (ca == 1)
-        c = s_part[lane & (FC_NW - 1)];
+        c = s_part[lane & (NW - 1)];
       else
         c = *on_cta(&s_pub[par], lane & (ca - 1));
       const unsigned h = __reduce_max_sync(0xffffffffu, c.hi);
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
       R wres = c.weight;
       for (int o = 1; o < ne; o <<= 1) wres = wres + sx(wres, o);
       if (j == n || l == 0u) break;  // l = 0: no open column
-      if (j >= 1 && (wres <= thr_w || best <= floor2)) break;
+      if (j >= 1 && (le_nn(wres, thr_w) || le_nn(best, floor2))) break;
       if (j >= cap) {
         fallback = true;
         break;
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
       const int op = p / cpb, lp = p - op * cpb;
       {
         const cx<R>* src = on_cta(W + (long)lp * n, op);
-        for (int i = tid; i < n; i += FC_NT) s_v[i] = src[i];
+        for (int i = tid; i < n; i += NT) s_v[i] = src[i];
       }
       __syncthreads();
       R nrm2 = best;
@@ -357,22 +359,20 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
           if (i < jl && gl == 1) s_c[i].im = h2;
         }
         __syncthreads();
-        // our part of Q c, two lanes per row (n <= 128) or one
-        const int sp = n <= FC_NT / 2 ? 2 : 1, row = tid / sp, half = tid - row * sp;
-        {
+        // our part of Q c, two lanes per row
+        for (int r0 = 0; r0 < n; r0 += NT / 2) {
+          const int row = r0 + tid / 2, half = tid & 1;
           Acc<R> re, im;
           if (row < n)
-            for (int i = half; i < jl; i += sp) {
+            for (int i = half; i < jl; i += 2) {
               const cx<R> x = s_c[i], q = W[(long)s_slot[i] * n + row];
               re.mac(x.re, q.re);
               re.mac(-x.im, q.im);
               im.mac(x.re, q.im);
               im.mac(x.im, q.re);
             }
-          if (sp == 2) {
-            re.add_from(re, 1);
-            im.add_from(im, 1);
-          }
+          re.add_from(re, 1);
+          im.add_from(im, 1);
           if (row < n && half == 0) {
             const cx<R> y = mk<R>(re.value(), im.value());
             if (ca == 1)
@@ -384,22 +384,25 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
         csync();
         if (ca > 1) {
           // our slice of rows: v - the CTAs' parts, ca lanes per row
-          const int sr = tid / ca, sc = tid - sr * ca, srow = k0c + sr;
-          cx<R> y = mk<R>(zero, zero);
-          if (sr < ncl) y = *on_cta(&s_y[srow], sc);
-          for (int o = 1; o < ca; o <<= 1) {
-            y.re = y.re + sx(y.re, o);
-            y.im = y.im + sx(y.im, o);
+          for (int s0 = 0; s0 < ncl; s0 += NT / ca) {
+            const int sr = s0 + tid / ca, sc = tid & (ca - 1), srow = k0c + sr;
+            if (s0 + (warp * 32) / ca >= ncl) break;  // no row for this warp
+            cx<R> y = mk<R>(zero, zero);
+            if (sr < ncl) y = *on_cta(&s_y[srow], sc);
+            for (int o = 1; o < ca; o <<= 1) {
+              y.re = y.re + sx(y.re, o);
+              y.im = y.im + sx(y.im, o);
+            }
+            if (sr < ncl && sc == 0) s_z[sr] = csub_r(s_v[srow], y);
           }
-          if (sr < ncl && sc == 0) s_z[sr] = csub_r(s_v[srow], y);
           csync();
-          for (int i = tid; i < n; i += FC_NT) s_v[i] = *on_cta(&s_z[i % cpb], i / cpb);
+          for (int i = tid; i < n; i += NT) s_v[i] = *on_cta(&s_z[i % cpb], i / cpb);
           __syncthreads();
         }
         const R prev = nrm2;
         {
           Acc<R> re, im;
-          for (int i = tid; i < n; i += FC_NT) {
+          for (int i = tid; i < n; i += NT) {
             const cx<R> x = s_v[i];
             re.mac(x.re, x.re);
             im.mac(x.im, x.im);
@@ -409,15 +412,15 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
           nrm2 = sa + sb;
         }
         if (tid == 0) flops += 16.0 * n * j;
-        if (nrm2 >= quarter * prev) break;
+        if (le_nn(quarter * prev, nrm2)) break;
       }
       // the pivot's true residual is at the rounding level: what the tracked norms still
       // show is rounding of earlier projections, and the range is complete
-      if (j >= 1 && nrm2 <= floor2) break;
+      if (j >= 1 && le_nn(nrm2, floor2)) break;
       if (j == 0) csync();  // every CTA has read the column that becomes q_0
       {
         const R inv = rsqrt_r(nrm2);
-        for (int i = tid; i < n; i += FC_NT) {
+        for (int i = tid; i < n; i += NT) {
           const cx<R> q = mk<R>(s_v[i].re * inv, s_v[i].im * inv);
           s_v[i] = q;
           if (rank == op) W[(long)lp * n + i] = q;
@@ -472,10 +475,10 @@ __global__ void __launch_bounds__(FC_NT, 1) k_range(EigDesc e, int* __restrict__
   };
   if (!usable) {  // G = 0 or non-finite entries: one unit vector
     if (rank == 0)
-      for (int i = tid; i < n; i += FC_NT) put(i, 0, i == 0 ? 1.0 : 0.0, 0.0);
+      for (int i = tid; i < n; i += NT) put(i, 0, i == 0 ? 1.0 : 0.0, 0.0);
     return;
   }
-  for (int x = tid; x < jl * n; x += FC_NT) {
+  for (int x = tid; x < jl * n; x += NT) {
     const int q = x / n, i = x - q * n;
     const cx<R> u = W[(long)s_slot[q] * n + i];
     put(i, s_idx[q], (double)u.re, (double)u.im);
@@ -501,7 +504,7 @@ cudaError_t launch_range(int n_max, const EigDesc& e, const int* d_dims, cudaStr
   cudaLaunchConfig_t cfg = {};
   const int c = range_ctas<R>(n_max);
   cfg.gridDim = dim3(c, members, 1);
-  cfg.blockDim = dim3(FC_NT, 1, 1);
+  cfg.blockDim = dim3(ClThreads<R>::v, 1, 1);
   cfg.dynamicSmemBytes = range_smem<R>(n_max);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
