@@ -32,10 +32,10 @@
 //
 // Measured on GB300, a cold G of rank r with weights over 1e-12 (against one CTA of 512
 // threads sweeping all columns, the kernel of the sizes above 256): FP64 n = 32, r = 16
-// 143 us (360), n = 64, r = 32 274 us (987), n = 128, r = 64 0.84 ms (4.47); double-float
-// 79 us (124), 270 us (348), 0.71 ms (2.25).  FP64 on four warps instead of eight, with its
-// comparisons off the FP64 pipe, is 31 us, 59 us and 0.10 ms of that: what every warp
-// computes for itself held the pipes for ~6,000 of a step's ~20,000 cycles.
+// 110 us (360), n = 64, r = 32 274 us (987), n = 128, r = 64 0.84 ms (4.47); double-float
+// 79 us (124), 239 us (348), 0.71 ms (2.25).  FP64 runs on four warps instead of eight, with
+// its comparisons off the FP64 pipe (n = 64 333 us and n = 128 0.94 ms on eight): what every
+// warp computes for itself held the pipes for ~6,000 of a step's ~20,000 cycles.
 //
 // R = double (the FP64 form) or df64 (the mixed forms).  G and U are FP64 in both.
 
@@ -58,16 +58,19 @@ struct RangeEps<df64> {
   static constexpr double v = 3.552713678800501e-15;  // 2^-48
 };
 
-constexpr int RB_LOCAL = 96;  // columns of one CTA at most
+constexpr int RB_LOCAL = 48;  // columns of one CTA at most
 
 // CTAs that work on a problem of size n (a power of two).  One CTA needs no exchange (three
 // barriers and four reads across CTAs, ~5,000 cycles a step) and takes ~5 n^2 cycles for the
-// sweep in FP64, an eighth of that in double-float: the lines lie where the two are equal,
-// for double-float where one CTA's shared memory ends.
+// sweep in FP64, an eighth of that in double-float.  The lines lie where the times of two
+// splits cross (r = n / 2): FP64 n = 24 92 us on one CTA and 88 on four, n = 32 143 on one,
+// 114 on four, 110 on eight, n = 64 337, 274, 270 on 4, 8, 16, n = 80 511 on eight, 432 on
+// 16; double-float n = 40 131 on one, 130 on eight, n = 64 270, 247, 239, 272 on 1, 2, 4, 8,
+// n = 80 530, 448, 368, 383, n = 128 724 on four, 707 on eight.
 template <typename R>
 __host__ __device__ inline int range_ctas(int n) {
-  if (std::is_same<R, double>::value) return n <= 32 ? 1 : n <= 64 ? 8 : 16;
-  return n <= 88 ? 1 : n <= 128 ? 8 : 16;
+  if (std::is_same<R, double>::value) return n <= 24 ? 1 : n <= 64 ? 8 : 16;
+  return n <= 48 ? 1 : n <= 96 ? 4 : n <= 128 ? 8 : 16;
 }
 
 // a pivot candidate (key: FP32 bits of the squared residual norm above the complement of
@@ -496,7 +499,7 @@ size_t range_smem(int n_max) {
   return (size_t)m * sizeof(cx<R>);
 }
 
-constexpr size_t RB_SMEM_LIMIT = 128 * 1024;  // double-float, n = 88 in one CTA: 121 KB
+constexpr size_t RB_SMEM_LIMIT = 80 * 1024;  // n = 256 over 16 CTAs: 64 KB
 
 template <typename R>
 cudaError_t launch_range(int n_max, const EigDesc& e, const int* d_dims, cudaStream_t s, double* prof,
