@@ -162,78 +162,6 @@ __global__ void __launch_bounds__(B_THREADS) k_osj_round(zd* X, int m, int n, zd
   }
 }
 
-// All sweeps of the row-wise one-sided Jacobi in one CTA (for moderate sizes):
-// warp w rotates the pairs w, w + 32, ... of each round; rounds are separated by
-// __syncthreads().  Stops after a sweep without rotation or after max_sweeps;
-// writes the number of sweeps run, or -1 when it stopped at the limit.
-constexpr int OSJ1_THREADS = 1024;
-__global__ void __launch_bounds__(OSJ1_THREADS) k_osj_all(zd* X, int m, int n, zd* T, const double* abs_thr_p,
-                                                        int max_sweeps, int* sweeps_out) {
-  __shared__ int s_rot;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nwarps = OSJ1_THREADS >> 5;
-  const int np = m + (m & 1);
-  const double abs_thr = *abs_thr_p;
-  const double rel = 2.220446049250313e-16 * fmax(8.0, 4.0 * sqrt((double)n));
-  int sw = 0;
-  for (; sw < max_sweeps; sw++) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
-    for (int round = 0; round < np - 1; round++) {
-      for (int t = warp; t < np / 2; t += nwarps) {
-        int p = rr_player_b(t, round, np), q = rr_player_b(np - 1 - t, round, np);
-        if (p > q) {
-          int x = p;
-          p = q;
-          q = x;
-        }
-        if (q >= m) continue;
-        zd* xp = X + (long)p * n;
-        zd* xq = X + (long)q * n;
-        double a = 0, b = 0, gr = 0, gi = 0;
-        for (int j = lane; j < n; j += 32) {
-          zd u = xp[j], v = xq[j];
-          a += u.re * u.re + u.im * u.im;
-          b += v.re * v.re + v.im * v.im;
-          gr += u.re * v.re + u.im * v.im;
-          gi += u.im * v.re - u.re * v.im;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          a += __shfl_xor_sync(0xffffffffu, a, o);
-          b += __shfl_xor_sync(0xffffffffu, b, o);
-          gr += __shfl_xor_sync(0xffffffffu, gr, o);
-          gi += __shfl_xor_sync(0xffffffffu, gi, o);
-        }
-        double x = sqrt(gr * gr + gi * gi);
-        if (!(x > 0.0 && x > rel * sqrt(a * b) && x > abs_thr)) continue;
-        double tau = (b - a) / (2 * x);
-        double tt = fabs(tau) > 1e100 ? 0.5 / tau : (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-        double c = 1.0 / sqrt(1.0 + tt * tt);
-        double s = tt * c;
-        zd sp = mk<double>(s * gr / x, s * gi / x);
-        for (int j = lane; j < n; j += 32) {
-          zd u = xp[j], v = xq[j];
-          xp[j] = csub(cscale(u, c), cmul(sp, v));
-          xq[j] = cadd(cmul(cconj(sp), u), cscale(v, c));
-        }
-        zd* tp = T + (long)p * m;
-        zd* tq = T + (long)q * m;
-        for (int j = lane; j < m; j += 32) {
-          zd u = tp[j], v = tq[j];
-          tp[j] = csub(cscale(u, c), cmul(sp, v));
-          tq[j] = cadd(cmul(cconj(sp), u), cscale(v, c));
-        }
-        if (lane == 0) atomicAdd(&s_rot, 1);
-      }
-      __syncthreads();
-    }
-    int nr = s_rot;
-    __syncthreads();
-    if (nr == 0) break;
-  }
-  if (threadIdx.x == 0) *sweeps_out = (sw < max_sweeps) ? sw + 1 : -1;
-}
-
 __global__ void k_abs_thr(const zd* X, long n, double* out) {
   __shared__ double sh[32];
   double acc = 0;
@@ -245,104 +173,6 @@ __global__ void k_abs_thr(const zd* X, long n, double* out) {
 __global__ void k_identity(zd* T, int m) {
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i < (long)m * m) T[i] = mk<double>((i / m) == (i % m) ? 1.0 : 0.0, 0.0);
-}
-
-// Row norms, sort, truncation rule, outputs.  One CTA; dynamic smem holds
-// w[m] (double) and perm[m] (int).  tall: X (m x n) holds the rotated rows of the conjugate
-// transpose of the matrix that was asked for, so its outputs are U (n x k) and R (k x m).
-__global__ void k_osj_finish(const zd* X, int m, int n, const zd* T, double tol, int cap, double gap, zd* U,
-                             int u_scale, zd* Rr, int r_unscale, int* k_out, double* s2_out, int tall) {
-  extern __shared__ unsigned char sm[];
-  double* w = (double*)sm;
-  double* ws = w + m;
-  int* perm = (int*)(ws + m);
-  __shared__ int s_k;
-  {  // row norms, one warp per row
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int i = warp; i < m; i += nw) {
-      double acc = 0;
-      for (int j = lane; j < n; j += 32) acc += cabs2(X[(long)i * n + j]);
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) w[i] = acc;
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    int r = 0;
-    for (int j = 0; j < m; j++)
-      if (w[j] > w[i] || (w[j] == w[i] && j < i)) r++;
-    perm[r] = i;
-  }
-  __syncthreads();
-  for (int r = threadIdx.x; r < m; r += blockDim.x) ws[r] = w[perm[r]];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // same rule as the step's truncation (relative discarded weight, cap, clusters)
-    double total = 0;
-    for (int i = 0; i < m; i++) total += ws[i];
-    int k = m;
-    if (!(total > 0)) {
-      k = 1;
-    } else {
-      double tail = 0;
-      while (k > 1 && tail + ws[k - 1] <= tol * total) {
-        tail += ws[k - 1];
-        k--;
-      }
-      if (cap > 0 && k > cap) k = cap;
-      if (k < m && sqrt(ws[k]) >= (1.0 - gap) * sqrt(ws[k - 1])) {
-        int j = k;
-        while (j < m && (cap <= 0 || j < cap) && sqrt(ws[j]) >= (1.0 - gap) * sqrt(ws[j - 1])) j++;
-        if (j < m && sqrt(ws[j]) >= (1.0 - gap) * sqrt(ws[j - 1])) {
-          j = k;
-          while (j > 1 && sqrt(ws[j]) >= (1.0 - gap) * sqrt(ws[j - 1])) j--;
-        }
-        k = j;
-      }
-      if (k < 1) k = 1;
-    }
-    s_k = k;
-    *k_out = k;
-    if (s2_out)
-      for (int i = 0; i < k; i++) s2_out[i] = ws[i];
-  }
-  __syncthreads();
-  int k = s_k;
-  if (tall) {
-    // A^dag = T^dag X, so A = X^dag T: U[i, j] = conj(X[perm_j, i]) / s_j, R[j, :] = s_j T[perm_j, :]
-    for (long x = threadIdx.x; x < (long)n * k; x += blockDim.x) {
-      int i = (int)(x / k), j = (int)(x % k);
-      zd v = cconj(X[(long)perm[j] * n + i]);
-      if (!u_scale) {
-        double s = sqrt(ws[j]);
-        v = (s > 0) ? cscale(v, 1.0 / s) : mk<double>(i == j ? 1.0 : 0.0, 0);
-      }
-      U[x] = v;
-    }
-    for (long x = threadIdx.x; x < (long)k * m; x += blockDim.x) {
-      int j = (int)(x / m), c = (int)(x % m);
-      zd v = T[(long)perm[j] * m + c];
-      Rr[x] = r_unscale ? v : cscale(v, sqrt(ws[j]));
-    }
-    return;
-  }
-  // U[i, j] = conj(T[perm_j, i]) * s_j^u_scale
-  for (long x = threadIdx.x; x < (long)m * k; x += blockDim.x) {
-    int i = (int)(x / k), j = (int)(x % k);
-    zd v = cconj(T[(long)perm[j] * m + i]);
-    if (u_scale) v = cscale(v, sqrt(ws[j]));
-    U[x] = v;
-  }
-  // R[j, :] = X[perm_j, :] / s_j^r_unscale
-  for (long x = threadIdx.x; x < (long)k * n; x += blockDim.x) {
-    int j = (int)(x / n), c = (int)(x % n);
-    zd v = X[(long)perm[j] * n + c];
-    if (r_unscale) {
-      double s = sqrt(ws[j]);
-      v = (s > 0) ? cscale(v, 1.0 / s) : mk<double>(0, 0);
-    }
-    Rr[x] = v;
-  }
 }
 
 // Built-in single-mode factors (Sec. II.B; charge basis Sec. VII).
@@ -447,84 +277,69 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
                    int r_unscale, int* k_out, int max_sweeps) {
   cudaStream_t s = ctx->stream;
   *U = *Rr = nullptr;
-  zd* T = nullptr;
   // The rows that are rotated are those of the matrix or of its conjugate transpose,
   // whichever are fewer: a sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so
   // the tall cores of a left-canonical sweep (4 D x D) cost a sixteenth (admission of an
-  // N = 64 cat, ~130 such solves: 248 ms before, 48 ms now).
+  // N = 64 cat, 135 such solves: 248 ms before, 48 with it).
   const int tall = m > n;
-  struct Xt {
+  struct Buf {  // freed on return unless handed over
     qlb_ctx* c;
-    zd* p = nullptr;
-    ~Xt() { dev_free(c, p); }
-  } xt{ctx};
+    void* p = nullptr;
+    ~Buf() { dev_free(c, p); }
+  } xt{ctx}, bt{ctx}, bc{ctx}, bu{ctx}, br{ctx};
+  qlb_status st;
   if (tall) {
-    qlb_status st = dev_alloc(ctx, (void**)&xt.p, sizeof(zd) * (size_t)m * n);
-    if (st) return st;
-    k_conj_transpose<<<nblk((long)m * n), 256, 0, s>>>(X, xt.p, m, n);
-    X = xt.p;
+    if ((st = dev_alloc(ctx, &xt.p, sizeof(zd) * (size_t)m * n))) return st;
+    k_conj_transpose<<<nblk((long)m * n), 256, 0, s>>>(X, (zd*)xt.p, m, n);
+    X = (zd*)xt.p;
     std::swap(m, n);
   }
-  int* d_cnt = nullptr;
-  int* d_k = nullptr;
-  qlb_status st;
-  if ((st = dev_alloc(ctx, (void**)&T, sizeof(zd) * (size_t)m * m))) return st;
-  if ((st = dev_alloc(ctx, (void**)&d_cnt, 4 * sizeof(double)))) {
-    dev_free(ctx, T);
+  // the factors are at most min(m, n) = m wide
+  if ((st = dev_alloc(ctx, &bt.p, sizeof(zd) * (size_t)m * m)) || (st = dev_alloc(ctx, &bc.p, 4 * sizeof(double))) ||
+      (st = dev_alloc(ctx, &bu.p, sizeof(zd) * (size_t)(tall ? n : m) * m)) ||
+      (st = dev_alloc(ctx, &br.p, sizeof(zd) * (size_t)m * (tall ? m : n))))
     return st;
+  zd* T = (zd*)bt.p;
+  int* d_cnt = (int*)bc.p;  // sweeps or rotations, then the kept count
+  const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, tall, (zd*)bu.p, (zd*)br.p, d_cnt + 1};
+  int h[2] = {0, 0};
+  if (osj_serves(m, n)) {
+    QLB_CUDA_TRY(launch_osj(X, m, n, T, max_sweeps, d_cnt, out, s));
+  } else {
+    double* d_thr = (double*)d_cnt + 1;
+    k_identity<<<nblk((long)m * m), 256, 0, s>>>(T, m);
+    k_abs_thr<<<1, 256, 0, s>>>(X, (long)m * n, d_thr);
+    const int np = m + (m & 1);
+    int conv = m <= 1;
+    for (int sw = 0; sw < max_sweeps && !conv; sw++) {
+      cudaMemsetAsync(d_cnt, 0, sizeof(int), s);
+      for (int r = 0; r < np - 1; r++) k_osj_round<<<np / 2, B_THREADS, 0, s>>>(X, m, n, T, np, r, d_cnt, d_thr);
+      int h_cnt = 0;
+      cudaMemcpyAsync(&h_cnt, d_cnt, sizeof(int), cudaMemcpyDeviceToHost, s);
+      QLB_CUDA_TRY(cudaStreamSynchronize(s));
+      conv = h_cnt == 0;
+    }
+    if (!conv) {
+      set_error("one-sided Jacobi SVD did not converge");
+      return QLB_ENOTCONV;
+    }
+    cudaMemsetAsync(d_cnt, 1, sizeof(int), s);  // converged
+    QLB_CUDA_TRY(launch_osj_finish(X, m, n, T, out, s));
   }
-  d_k = d_cnt + 1;
-  double* d_thr = (double*)d_cnt + 1;
-  k_identity<<<nblk((long)m * m), 256, 0, s>>>(T, m);
-  k_abs_thr<<<1, 256, 0, s>>>(X, (long)m * n, d_thr);
-  int np = m + (m & 1);
-  bool conv = (m <= 1);
-  if (!conv && (long)n <= 16384) {
-    // moderate rows: every sweep in one launch
-    int* d_sw = d_cnt;
-    k_osj_all<<<1, OSJ1_THREADS, 0, s>>>(X, m, n, T, d_thr, max_sweeps, d_sw);
-    int h_sw = 0;
-    cudaMemcpyAsync(&h_sw, d_sw, sizeof(int), cudaMemcpyDeviceToHost, s);
-    QLB_CUDA_TRY(cudaStreamSynchronize(s));
-    conv = h_sw > 0;
-    max_sweeps = 0;  // skip the multi-launch loop below
-  }
-  for (int sw = 0; sw < max_sweeps && !conv; sw++) {
-    cudaMemsetAsync(d_cnt, 0, sizeof(int), s);
-    for (int r = 0; r < np - 1; r++) k_osj_round<<<np / 2, B_THREADS, 0, s>>>(X, m, n, T, np, r, d_cnt, d_thr);
-    int h_cnt = 0;
-    cudaMemcpyAsync(&h_cnt, d_cnt, sizeof(int), cudaMemcpyDeviceToHost, s);
-    QLB_CUDA_TRY(cudaStreamSynchronize(s));
-    conv = (h_cnt == 0);
-  }
-  if (!conv) {
-    dev_free(ctx, T);
-    dev_free(ctx, d_cnt);
-    set_error("one-sided Jacobi SVD did not converge");
-    return QLB_ENOTCONV;
-  }
-  // outputs at most min(m, n) wide... allocate for m (k <= m)
-  int kmax = m;
-  if ((st = dev_alloc(ctx, (void**)U, sizeof(zd) * (size_t)(tall ? n : m) * kmax)) ||
-      (st = dev_alloc(ctx, (void**)Rr, sizeof(zd) * (size_t)kmax * (tall ? m : n)))) {
-    dev_free(ctx, T);
-    dev_free(ctx, d_cnt);
-    dev_free(ctx, *U);
-    *U = nullptr;
-    return st;
-  }
-  size_t sm = (size_t)m * (2 * sizeof(double) + sizeof(int));
-  if (sm > 48 * 1024) cudaFuncSetAttribute(k_osj_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_osj_finish<<<1, 256, sm, s>>>(X, m, n, T, tol, cap, 1e-10, *U, u_scale, *Rr, r_unscale, d_k, nullptr, tall);
-  int hk = 0;
-  cudaMemcpyAsync(&hk, d_k, sizeof(int), cudaMemcpyDeviceToHost, s);
+  cudaMemcpyAsync(h, d_cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);
-  dev_free(ctx, T);
-  dev_free(ctx, d_cnt);
   if (e != cudaSuccess) {
     set_error(std::string("svd finish: ") + cudaGetErrorString(e));
     return QLB_EDEVICE;
   }
+  if (h[0] <= 0) {
+    set_error("one-sided Jacobi SVD did not converge");
+    return QLB_ENOTCONV;
+  }
+  const int hk = h[1];
+  *U = (zd*)bu.p;
+  *Rr = (zd*)br.p;
+  bu.p = br.p = nullptr;
   *k_out = hk;
   return QLB_OK;
 }

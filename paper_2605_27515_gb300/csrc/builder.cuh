@@ -65,6 +65,20 @@ template <typename R>
 cudaError_t launch_zipqr_group(int n_max, const EigDesc* d_grp, int S, cudaStream_t s, double* prof);
 void init_tc_attributes();
 
+// one-sided Jacobi SVD of the builder (kernels_osj.cu).  tall: X holds the rows of the
+// conjugate transpose of the matrix that was asked for, so U is n x k and Rr k x m
+struct OsjOut {
+  double tol, gap;
+  int cap, u_scale, r_unscale, tall;
+  zd *U, *Rr;
+  int* k_out;
+};
+bool osj_serves(int m, int n);
+// all sweeps on the rows of X (m x n; may be overwritten, like T, m x m) and the factors
+cudaError_t launch_osj(zd* X, int m, int n, zd* T, int max_sweeps, int* sweeps_out, const OsjOut& out, cudaStream_t s);
+// the factors alone, from rotated rows X and the rotations T
+cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, const OsjOut& out, cudaStream_t s);
+void init_osj_attributes();
 qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** U, int u_scale, zd** Rr,
                    int r_unscale, int* k_out, int max_sweeps);
 qlb_status tt_svd(qlb_ctx* ctx, zd* T, int L, int P, double tol, int cap, std::vector<zd*>& cores,
