@@ -17,7 +17,9 @@ namespace qlb {
 
 // ------------------------------------------------------------------ memory
 
-qlb_status dev_alloc(qlb_ctx* ctx, void** p, size_t bytes) {
+// dev_alloc without the wait, for buffers that only the context stream touches until the
+// caller has synchronised it: an SVD takes four or five, and the waits were ~5 us each.
+qlb_status dev_alloc_queued(qlb_ctx* ctx, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
   if (ctx->opt.hbm_budget && ctx->mem_held + bytes > ctx->opt.hbm_budget) {
@@ -25,13 +27,7 @@ qlb_status dev_alloc(qlb_ctx* ctx, void** p, size_t bytes) {
               std::to_string(ctx->opt.hbm_budget) + " bytes)");
     return QLB_ENOMEM;
   }
-  // Stream-ordered allocation from the device's memory pool: unlike cudaMalloc /
-  // cudaFree it never synchronises the whole device, so admitting or retiring one
-  // state does not drain the steps other states have in flight.  The buffer is
-  // complete when the context stream is, which the synchronisation below ensures
-  // before any other stream touches it.
   cudaError_t e = cudaMallocAsync(p, bytes, ctx->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {
     *p = nullptr;
     set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
@@ -40,6 +36,24 @@ qlb_status dev_alloc(qlb_ctx* ctx, void** p, size_t bytes) {
   ctx->mem_held += bytes;
   ctx->n_allocs++;
   g_alloc_sizes()[*p] = std::make_pair(bytes, ctx);
+  return QLB_OK;
+}
+
+// Stream-ordered allocation from the device's memory pool: unlike cudaMalloc /
+// cudaFree it never synchronises the whole device, so admitting or retiring one
+// state does not drain the steps other states have in flight.  The buffer is
+// complete when the context stream is, which the synchronisation below ensures
+// before any other stream touches it.
+qlb_status dev_alloc(qlb_ctx* ctx, void** p, size_t bytes) {
+  qlb_status st = dev_alloc_queued(ctx, p, bytes);
+  if (st) return st;
+  cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) {
+    dev_free(ctx, *p);
+    *p = nullptr;
+    set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
+    return QLB_ENOMEM;
+  }
   return QLB_OK;
 }
 
@@ -289,15 +303,15 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   } xt{ctx}, bt{ctx}, bc{ctx}, bu{ctx}, br{ctx};
   qlb_status st;
   if (tall) {
-    if ((st = dev_alloc(ctx, &xt.p, sizeof(zd) * (size_t)m * n))) return st;
+    if ((st = dev_alloc_queued(ctx, &xt.p, sizeof(zd) * (size_t)m * n))) return st;
     k_conj_transpose<<<nblk((long)m * n), 256, 0, s>>>(X, (zd*)xt.p, m, n);
     X = (zd*)xt.p;
     std::swap(m, n);
   }
   // the factors are at most min(m, n) = m wide
-  if ((st = dev_alloc(ctx, &bt.p, sizeof(zd) * (size_t)m * m)) || (st = dev_alloc(ctx, &bc.p, 4 * sizeof(double))) ||
-      (st = dev_alloc(ctx, &bu.p, sizeof(zd) * (size_t)(tall ? n : m) * m)) ||
-      (st = dev_alloc(ctx, &br.p, sizeof(zd) * (size_t)m * (tall ? m : n))))
+  if ((st = dev_alloc_queued(ctx, &bt.p, sizeof(zd) * (size_t)m * m)) || (st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double))) ||
+      (st = dev_alloc_queued(ctx, &bu.p, sizeof(zd) * (size_t)(tall ? n : m) * m)) ||
+      (st = dev_alloc_queued(ctx, &br.p, sizeof(zd) * (size_t)m * (tall ? m : n))))
     return st;
   zd* T = (zd*)bt.p;
   int* d_cnt = (int*)bc.p;  // sweeps or rotations, then the kept count
@@ -513,7 +527,7 @@ qlb_status mpo_compress(qlb_ctx* ctx, Mpo& W, double tol, int cap) {
     // core_{i+1} <- Rr (k x n) * core_{i+1} (n x 4 D_{i+2})
     int n2 = 4 * W.D[i + 2];
     zd* nc;
-    if ((st = dev_alloc(ctx, (void**)&nc, sizeof(zd) * (size_t)k * n2))) return st;
+    if ((st = dev_alloc_queued(ctx, (void**)&nc, sizeof(zd) * (size_t)k * n2))) return st;
     GemmDesc g{};
     g.A = Rr;
     g.B = W.core[i + 1];
@@ -546,7 +560,7 @@ qlb_status mpo_compress(qlb_ctx* ctx, Mpo& W, double tol, int cap) {
     W.core[i] = Vh;  // [k][4][D_{i+1}]
     int m2 = W.D[i - 1] * 4;
     zd* nc;
-    if ((st = dev_alloc(ctx, (void**)&nc, sizeof(zd) * (size_t)m2 * k))) return st;
+    if ((st = dev_alloc_queued(ctx, (void**)&nc, sizeof(zd) * (size_t)m2 * k))) return st;
     GemmDesc g{};
     g.A = W.core[i - 1];
     g.B = US;

@@ -10,6 +10,7 @@
 namespace qlb {
 
 qlb_status dev_alloc(qlb_ctx* ctx, void** p, size_t bytes);
+qlb_status dev_alloc_queued(qlb_ctx* ctx, void** p, size_t bytes);
 void dev_free(qlb_ctx* ctx, void* p);
 std::map<void*, std::pair<size_t, qlb_ctx*>>& g_alloc_sizes();
 
