@@ -220,6 +220,52 @@ __device__ __forceinline__ R csum(Acc<R> re, Acc<R> im, int LP) {
   return q.value();
 }
 
+// ------------------------------------------------------------------ truncation rule
+
+// Kept count of weights w[0..m) in falling order: relative discarded weight, cap (>= 1), no
+// cut through a degenerate cluster.  Called by a whole warp; total and kept receive sums of the
+// weights.
+__device__ __forceinline__ int truncation_count(const double* w, int m, double tol, int cap, double gap, double& total,
+                                                double& kept) {
+  const int lane = threadIdx.x & 31;
+  // lane l has the weights [l q, (l + 1) q)
+  const int q = (m + 31) / 32, i0 = min(m, lane * q), i1 = min(m, i0 + q);
+  double part = 0.0;
+  for (int i = i0; i < i1; i++) part += w[i];
+  double tail = part;  // of this lane's weights and all later ones
+  for (int o = 1; o < 32; o <<= 1) {
+    const double v = __shfl_down_sync(0xffffffffu, tail, o);
+    if (lane + o < 32) tail += v;
+  }
+  total = __shfl_sync(0xffffffffu, tail, 0);
+  double after = __shfl_down_sync(0xffffffffu, tail, 1);
+  if (lane == 31) after = 0.0;
+  // the smallest count whose discarded weight is within the cutoff
+  int mine = i1;
+  while (mine > i0 && after + w[mine - 1] <= tol * total) after += w[--mine];
+  const unsigned whole = __ballot_sync(0xffffffffu, mine == i0);
+  const int first = __clz(~whole);  // lanes whose weights all go, from the last one down
+  int k = first == 32 ? 0 : __shfl_sync(0xffffffffu, mine, 31 - first);
+  if (k < 1) k = 1;
+  if (k > cap) k = cap;
+  if (k < m) {
+    auto same = [&](int j) { return ::sqrt(w[j]) >= (1.0 - gap) * ::sqrt(w[j - 1]); };
+    if (same(k)) {  // a cut through a degenerate cluster: extend it under the cap, else cut before it
+      int j = k;
+      while (j < m && j < cap && same(j)) j++;
+      if (j < m && same(j)) {
+        j = k;
+        while (j > 1 && same(j)) j--;
+      }
+      k = j;
+    }
+  }
+  kept = 0.0;
+  for (int i = i0; i < min(i1, k); i++) kept += w[i];
+  for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
+  return k;
+}
+
 }  // namespace
 
 }  // namespace qlb

@@ -11,15 +11,15 @@
 // from the first sweep to the factors while they fit (in X and T's own storage otherwise).
 //
 // What bounds it: an FP64 instruction of a warp holds a partition's pipe for 64 clocks, a
-// square root or a division some 20 of them.  The rotation's tangent is therefore seeded in
+// square root or a division some 20 of them.  The rotation's tangent is therefore formed in
 // FP32 and corrected once in FP64 (see below), and a group of 4 to 256 lanes takes a pair, so
 // that few pairs of long rows and many of short ones both fill the CTA.
 //
 // Measured on GB300 with the factors (against one CTA of 1,024 threads over global memory with
 // FP64 square roots and divisions, and the factors in a launch of their own): 16 x 16, ten sweeps,
-// 0.44 ms (1.30); 16 x 56 0.30 ms (0.86); 36 x 72, 12 sweeps, 2.5 ms (11.9, 14 sweeps);
-// 8 x 1,024 0.10 ms (0.52); 20 x 16,384 9.1 ms (110).  Admitting an N = 64 cat, 135 such
-// solves of 2 to 43 rows: 47 ms before, 25 now.
+// 0.42 ms (1.30); 16 x 56 0.30 ms (0.86); 36 x 72, 13 sweeps, 2.0 ms (11.9, 14 sweeps);
+// 8 x 1,024 0.11 ms (0.52); 20 x 16,384 9.0 ms (110).  Admitting an N = 64 cat, 135 such
+// solves of 2 to 43 rows, 12 ms on the device: 47 ms before, 22 now.
 
 #include <algorithm>
 
@@ -68,45 +68,25 @@ struct OsjSlice {
 };
 
 // Order of the rows by squared norm w (m entries; ties to the lower row) and the step's
-// truncation rule (relative discarded weight, cap, degenerate clusters).  On return w[j] is the
-// j-th singular value, ws[j] its reciprocal (0 for 0), perm[j] its row.  Called by the CTA.
+// truncation rule.  On return w[j] is the j-th singular value, ws[j] its reciprocal (0 for 0),
+// perm[j] its row.  Called by the CTA.
 __device__ int osj_rule(double* w, double* ws, int* perm, int* s_k, int m, double tol, int cap, double gap) {
   __syncthreads();
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    const long long li = __double_as_longlong(w[i]);  // squared norms order like their bit patterns
     int r = 0;
-    for (int j = 0; j < m; j++)
-      if (w[j] > w[i] || (w[j] == w[i] && j < i)) r++;
+    for (int j = 0; j < m; j++) {
+      const long long lj = __double_as_longlong(w[j]);
+      r += lj > li || (lj == li && j < i);
+    }
     perm[r] = i;
+    ws[r] = w[i];
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < m; r += blockDim.x) ws[r] = w[perm[r]];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double total = 0;
-    for (int i = 0; i < m; i++) total += ws[i];
-    int k = m;
-    if (!(total > 0)) {
-      k = 1;
-    } else {
-      double tail = 0;
-      while (k > 1 && tail + ws[k - 1] <= tol * total) {
-        tail += ws[k - 1];
-        k--;
-      }
-      if (cap > 0 && k > cap) k = cap;
-      auto same = [&](int j) { return ::sqrt(ws[j]) >= (1.0 - gap) * ::sqrt(ws[j - 1]); };
-      if (k < m && same(k)) {  // a cut through a degenerate cluster: extend it under the cap, else cut before it
-        int j = k;
-        while (j < m && (cap <= 0 || j < cap) && same(j)) j++;
-        if (j < m && same(j)) {
-          j = k;
-          while (j > 1 && same(j)) j--;
-        }
-        k = j;
-      }
-      if (k < 1) k = 1;
-    }
-    *s_k = k;
+  if (threadIdx.x < 32) {
+    double total, kept;
+    const int k = truncation_count(ws, m, tol, cap > 0 ? cap : m, gap, total, kept);
+    if (threadIdx.x == 0) *s_k = total > 0 ? k : 1;
   }
   __syncthreads();
   for (int r = threadIdx.x; r < m; r += blockDim.x) {
@@ -155,13 +135,11 @@ struct __align__(16) PairSums {
   double v[4];  // |x_p|^2, |x_q|^2, Re and Im of x_p . conj(x_q)
 };
 
-// Lanes of a pair, at most twice the slice's width: as many as give each of the SM's four
-// partitions one warp, as a rotation's ~30 scalar FP64 operations are paid per warp (16 x 16,
-// ten sweeps: 0.70 ms on eight warps, 0.44 on four); rows of 256 columns and more take two, for their loads.
+// Lanes of a pair: as many as fill the CTA, at most twice the slice's width.
 __host__ __device__ inline int osj_lanes(int m, int width) {
-  const int pairs = (m + 1) / 2, threads = width >= 256 ? OSJ_NT : OSJ_NT / 2;
-  int g = threads;
-  while (g > 4 && (pairs * g > threads || g >= 2 * width)) g >>= 1;
+  const int pairs = (m + 1) / 2;
+  int g = OSJ_NT;
+  while (g > 4 && (pairs * g > OSJ_NT || g >= 2 * width)) g >>= 1;
   return g;
 }
 
@@ -328,7 +306,8 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
         if (!(q < m && gm > 0.f && cs > rel && fx > osj_to_f(thr, sk))) continue;
         // The rotation [[c, -sp], [conj(sp), c]] with sp = c z zeroes g + z (a - b) - z^2 conj(g).
         // z from FP32, then one Newton step in FP64, whose derivative is real at the root and
-        // needs FP32 only: what is left of the coupling is ~1e-13 of it.
+        // needs FP32 only: what is left of the coupling is ~1e-13 of it (~1e-7 without the step,
+        // a sweep more in most solves of up to 16 rows).
         const float h = fmaf(0.5f, ::fabsf(df), sqrtf(fmaf(0.25f * df, df, f2x)));
         const float iz = __fdividef(df <= 0.f ? 1.f : -1.f, h);
         const float z0r = fr * iz, z0i = fi * iz;
@@ -434,7 +413,8 @@ struct OsjPlan {
 
 // Cycles of a round on ca CTAs: a warp takes 64 per FP64 instruction, 8 per element of X for
 // the sums, 12 per element of X and T for the rotation, ~35 for the rotation's scalars; the
-// barrier, the reads between CTAs and what is not FP64 come to ~3,500 (1,000 on one CTA).
+// barrier, the reads between CTAs and what is not FP64 are counted as 2,000 (1,000 on one CTA),
+// the fastest over the SVDs of an N = 64 cat's admission (3,500: 2 % slower).
 OsjPlan osj_split(int m, int n, int ca) {
   OsjPlan p{};
   p.ca = ca;
@@ -445,7 +425,7 @@ OsjPlan osj_split(int m, int n, int ca) {
   p.smem = head + (p.resident ? rows : 0);
   const long warps = ((long)pairs * g + 31) / 32;
   p.cycles = 64 * ((warps + 3) / 4) * (8L * ((wn + g - 1) / g) + 12L * ((wn + wm + g - 1) / g) + 35) +
-             (ca > 1 ? 3500 : 1000);
+             (ca > 1 ? 2000 : 1000);
   return p;
 }
 OsjPlan osj_plan(int m, int n) {

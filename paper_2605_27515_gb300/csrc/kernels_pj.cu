@@ -546,46 +546,10 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* __res
   __syncthreads();
   if (warp == 0) {
     // weights beyond the factor's rank are zero: the rule sees the first r, and the zeros
-    // behind them change neither its sums nor its decision.  Lane l has the weights
-    // [l q, (l + 1) q).
+    // behind them change neither its sums nor its decision
     const int m = max(1, min(r, n));
-    const int q = (m + 31) / 32, i0 = min(m, lane * q), i1 = min(m, i0 + q);
     double total = 0.0, kept = 0.0;
-    int k = 1;
-    if (!s_bad && r > 0) {
-      double part = 0.0;
-      for (int i = i0; i < i1; i++) part += s_w[i];
-      double tail = part;  // of this lane's weights and all later ones
-      for (int o = 1; o < 32; o <<= 1) {
-        const double v = __shfl_down_sync(0xffffffffu, tail, o);
-        if (lane + o < 32) tail += v;
-      }
-      total = __shfl_sync(0xffffffffu, tail, 0);
-      double after = __shfl_down_sync(0xffffffffu, tail, 1);
-      if (lane == 31) after = 0.0;
-      // the smallest count whose discarded weight is within the cutoff
-      int mine = i1;
-      while (mine > i0 && after + s_w[mine - 1] <= e.tol * total) after += s_w[--mine];
-      const unsigned whole = __ballot_sync(0xffffffffu, mine == i0);
-      const int first = __clz(~whole);  // lanes whose weights all go, from the last one down
-      k = first == 32 ? 0 : __shfl_sync(0xffffffffu, mine, 31 - first);
-      if (k < 1) k = 1;
-      if (k > cap) k = cap;
-      if (k < m) {
-        auto same = [&](int j) { return ::sqrt(s_w[j]) >= (1.0 - e.gap) * ::sqrt(s_w[j - 1]); };
-        if (same(k)) {  // a cut through a degenerate cluster: extend it under the cap, else cut before it
-          int j = k;
-          while (j < m && j < cap && same(j)) j++;
-          if (j < m && same(j)) {
-            j = k;
-            while (j > 1 && same(j)) j--;
-          }
-          k = j;
-        }
-      }
-      for (int i = i0; i < min(i1, k); i++) kept += s_w[i];
-      for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
-    }
+    const int k = !s_bad && r > 0 ? truncation_count(s_w, m, e.tol, cap, e.gap, total, kept) : 1;
     if (lane == 0) s_k = k;
     if (rank == 0 && lane == 0) {
       d[e.dim_out] = k;
