@@ -128,7 +128,7 @@ struct GemmPlan {
 
 // One launch's work items with TS x TS tiles.
 template <typename Cm, int TS>
-__device__ void gemm_items(const GemmDesc& g, const int* __restrict__ d, const GemmPlan& P, int gnom, unsigned char* sm,
+__device__ void gemm_items(const GemmDesc& g, const int* d, const GemmPlan& P, int gnom, unsigned char* sm,
                           int* s_last) {
   constexpr int SL = G_THREADS / (TS * TS);  // K slices of a chunk (1 or 4)
   constexpr int LD = TS + 1;
@@ -259,7 +259,7 @@ __device__ void gemm_items(const GemmDesc& g, const int* __restrict__ d, const G
 // Cm: the type the products are formed and summed in (double, or double-float in the
 // mixed forms)
 template <typename Cm, bool GRP>
-__global__ void __launch_bounds__(G_THREADS, 3) k_gemm(const GemmDesc g_in, const int* __restrict__ d_in, double* prof,
+__global__ void __launch_bounds__(G_THREADS, 3) k_gemm(const GemmDesc g_in, const int* d_in, double* prof,
                                                        const GemmDesc* __restrict__ grp) {
   // grouped launch: this CTA works on member blockIdx.y, whose descriptor (and dims)
   // come from the group's table (kept in shared memory, not registers); the tile and the K
@@ -273,7 +273,9 @@ __global__ void __launch_bounds__(G_THREADS, 3) k_gemm(const GemmDesc g_in, cons
     __syncthreads();
   }
   const GemmDesc& g = GRP ? s_g : g_in;
-  const int* __restrict__ d = GRP ? s_g.dims : d_in;
+  const int* d = GRP ? s_g.dims : d_in;
+  after_previous();
+  let_next_start();
   const int gnom = g.split_grid > 0 ? g.split_grid : (int)gridDim.x;
   GemmPlan P;
   P.m = dev_eval(g.m, d);
@@ -348,10 +350,8 @@ cudaError_t launch_gemm(const GemmDesc& g, const int* d_dims, cudaStream_t s, do
   const int grid = g.ws ? full : (int)std::min<long>(planned, full);
   gg.split_grid = full;
   if (g.df64)
-    k_gemm<df64, false><<<grid, G_THREADS, 0, s>>>(gg, d_dims, prof, nullptr);
-  else
-    k_gemm<double, false><<<grid, G_THREADS, 0, s>>>(gg, d_dims, prof, nullptr);
-  return cudaGetLastError();
+    return launch_after(k_gemm<df64, false>, dim3(grid), G_THREADS, s, gg, d_dims, prof, nullptr);
+  return launch_after(k_gemm<double, false>, dim3(grid), G_THREADS, s, gg, d_dims, prof, nullptr);
 }
 
 // The same GEMM of S states in one launch: grid (per-member CTAs, S).  Every member
@@ -365,10 +365,8 @@ cudaError_t launch_gemm_group(const GemmDesc* d_grp, int S, int use_df, cudaStre
   const int per = std::max(8, std::min(full, (full + S - 1) / S));
   GemmDesc dummy{};
   if (use_df)
-    k_gemm<df64, true><<<dim3(per, S), G_THREADS, 0, s>>>(dummy, nullptr, prof, d_grp);
-  else
-    k_gemm<double, true><<<dim3(per, S), G_THREADS, 0, s>>>(dummy, nullptr, prof, d_grp);
-  return cudaGetLastError();
+    return launch_after(k_gemm<df64, true>, dim3(per, S), G_THREADS, s, dummy, nullptr, prof, d_grp);
+  return launch_after(k_gemm<double, true>, dim3(per, S), G_THREADS, s, dummy, nullptr, prof, d_grp);
 }
 
 }  // namespace qlb

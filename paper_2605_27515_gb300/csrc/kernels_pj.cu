@@ -267,10 +267,11 @@ struct __align__(16) PjSweep {
 // ------------------------------------------------------------------ the kernel
 
 template <typename R, bool GRP>
-__global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* __restrict__ d, double* prof,
+__global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, double* prof,
                                              const EigDesc* __restrict__ grp) {
   constexpr int NT = ClThreads<R>::v, NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if constexpr (GRP) {  // grouped launch: one cluster per member (blockIdx.y; the cluster spans x)
     e = grp[blockIdx.y];
     d = e.dims;
@@ -529,6 +530,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* __res
   csync();
   for (int i = tid; i < ns; i += NT) s_lam[i] = *on_cta(&s_own[i % nc], i / nc);
   csync();  // the last access to another CTA's shared memory
+  let_next_start();
   if (tid == 0) s_bad = any_bad ? 1 : 0;
   __syncthreads();
   for (int i = tid; i < ns; i += NT) {
@@ -632,13 +634,15 @@ cudaError_t launch_pj(int n_max, const EigDesc& e, const int* d_dims, cudaStream
   cfg.blockDim = dim3(ClThreads<R>::v, 1, 1);
   cfg.dynamicSmemBytes = pj_smem<R>(n_max);
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = c;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   if (grp) return cudaLaunchKernelEx(&cfg, k_pj<R, true>, e, (int*)d_dims, prof, grp);
   return cudaLaunchKernelEx(&cfg, k_pj<R, false>, e, (int*)d_dims, prof, grp);
 }

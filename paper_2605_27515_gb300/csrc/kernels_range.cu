@@ -82,10 +82,11 @@ struct __align__(16) Candidate {
 };
 
 template <typename R, bool GRP>
-__global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* __restrict__ d, double* prof,
+__global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d, double* prof,
                                                  const EigDesc* __restrict__ grp) {
   constexpr int NT = ClThreads<R>::v, NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if constexpr (GRP) {  // grouped launch: one cluster per member (blockIdx.y; the cluster spans x)
     e = grp[blockIdx.y];
     d = e.dims;
@@ -444,6 +445,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* __
     }
   }
   csync();  // nobody reads another CTA's shared memory any more
+  let_next_start();
   const int r = usable ? j : 1;
   if (rank == 0 && tid == 0) {
     if (cb.lost && e.err) atomicOr(e.err, 4);
@@ -510,13 +512,15 @@ cudaError_t launch_range(int n_max, const EigDesc& e, const int* d_dims, cudaStr
   cfg.blockDim = dim3(ClThreads<R>::v, 1, 1);
   cfg.dynamicSmemBytes = range_smem<R>(n_max);
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = c;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   if (grp) return cudaLaunchKernelEx(&cfg, k_range<R, true>, e, (int*)d_dims, prof, grp);
   return cudaLaunchKernelEx(&cfg, k_range<R, false>, e, (int*)d_dims, prof, grp);
 }

@@ -161,6 +161,35 @@ struct EigDesc {
   void* work;
 };
 
+// ------------------------------------------------------------------ dependent launches
+//
+// The kernels of a step and of an expectation value depend each on the one before.  They are
+// launched while it still runs (programmatic stream serialization; a programmatic edge
+// in a captured graph): such a kernel's CTAs take their places and wait in after_previous,
+// which returns when the launch before is complete and its writes are visible.  Nothing that
+// an earlier launch writes is read before it, nor through the read-only path (no const
+// __restrict__ on it).  let_next_start is the predecessor's side: the next launch may
+// take its places.
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // ------------------------------------------------------------------ error plumbing
 
 void set_error(const std::string& msg);

@@ -65,13 +65,25 @@ __device__ void step_begin_body(const StepBeginArgs& a) {
     }
   }
 }
-__global__ void k_step_begin(StepBeginArgs a) { step_begin_body(a); }
-__global__ void k_step_begin_grp(const StepBeginArgs* __restrict__ a) { step_begin_body(a[blockIdx.y]); }
+__global__ void k_step_begin(StepBeginArgs a) {
+  after_previous();
+  let_next_start();
+  step_begin_body(a);
+}
+__global__ void k_step_begin_grp(const StepBeginArgs* __restrict__ a) {
+  after_previous();
+  let_next_start();
+  step_begin_body(a[blockIdx.y]);
+}
 
 __global__ void k_step_end(StepEndArgs a) {
+  after_previous();
+  let_next_start();
   if (a.count && threadIdx.x == 0 && blockIdx.x == 0) (*a.step)++;
 }
 __global__ void k_step_end_grp(const StepEndArgs* __restrict__ a) {
+  after_previous();
+  let_next_start();
   const StepEndArgs x = a[blockIdx.y];
   if (x.count && threadIdx.x == 0 && blockIdx.x == 0) (*x.step)++;
 }
@@ -88,8 +100,16 @@ __device__ void copy_body(const CopyArgs& c) {
   for (long x = blockIdx.x * (long)blockDim.x + threadIdx.x; x < n; x += (long)gridDim.x * blockDim.x)
     c.dst[x] = c.src[x];
 }
-__global__ void k_copy(CopyArgs c) { copy_body(c); }
-__global__ void k_copy_grp(const CopyArgs* __restrict__ c) { copy_body(c[blockIdx.y]); }
+__global__ void k_copy(CopyArgs c) {
+  after_previous();
+  let_next_start();
+  copy_body(c);
+}
+__global__ void k_copy_grp(const CopyArgs* __restrict__ c) {
+  after_previous();
+  let_next_start();
+  copy_body(c[blockIdx.y]);
+}
 
 __global__ void k_sum_abs2(const zd* p, DimExpr cnt, const int* d, double* out) {
   __shared__ double sh[32];
@@ -331,7 +351,7 @@ static qlb_status copy(qlb_state* st, zd* dst, const zd* src, DimExpr cnt, long 
   }
   cudaEvent_t a;
   prof_before(ctx, st->stream, QLB_K_OTHER, &a);
-  k_copy<<<nblk(max_n), 256, 0, st->stream>>>(c);
+  QLB_CUDA_TRY(launch_after(k_copy, dim3(nblk(max_n)), 256, st->stream, c));
   prof_after(ctx, st->stream, QLB_K_OTHER, a);
   QLB_CUDA_TRY(cudaGetLastError());
   return QLB_OK;
@@ -935,7 +955,7 @@ qlb_status enqueue_step(qlb_state* st, const Kraus& K, bool count_step) {
     } else {
       cudaEvent_t a;
       prof_before(ctx, st->stream, QLB_K_OTHER, &a);
-      k_step_begin<<<nblk(n0), 256, 0, st->stream>>>(ba);
+      QLB_CUDA_TRY(launch_after(k_step_begin, dim3(nblk(n0)), 256, st->stream, ba));
       prof_after(ctx, st->stream, QLB_K_OTHER, a);
       QLB_CUDA_TRY(cudaGetLastError());
     }
@@ -1048,7 +1068,7 @@ qlb_status enqueue_step(qlb_state* st, const Kraus& K, bool count_step) {
     } else {
       cudaEvent_t a;
       prof_before(ctx, st->stream, QLB_K_OTHER, &a);
-      k_step_end<<<1, 32, 0, st->stream>>>(ea);
+      QLB_CUDA_TRY(launch_after(k_step_end, dim3(1), 32, st->stream, ea));
       prof_after(ctx, st->stream, QLB_K_OTHER, a);
       QLB_CUDA_TRY(cudaGetLastError());
     }
@@ -1428,16 +1448,13 @@ static qlb_status group_capture(GroupExec& gx, const std::vector<qlb_state*>& ms
     launches++;
     switch (r0.kind) {
       case REC_BEGIN:
-        k_step_begin_grp<<<dim3(nblk(maxn), S), 256, 0, gs>>>((const StepBeginArgs*)t);
-        e = cudaGetLastError();
+        e = launch_after(k_step_begin_grp, dim3(nblk(maxn), S), 256, gs, (const StepBeginArgs*)t);
         break;
       case REC_END:
-        k_step_end_grp<<<dim3(1, S), 32, 0, gs>>>((const StepEndArgs*)t);
-        e = cudaGetLastError();
+        e = launch_after(k_step_end_grp, dim3(1, S), 32, gs, (const StepEndArgs*)t);
         break;
       case REC_COPY:
-        k_copy_grp<<<dim3(nblk(maxn), S), 256, 0, gs>>>((const CopyArgs*)t);
-        e = cudaGetLastError();
+        e = launch_after(k_copy_grp, dim3(nblk(maxn), S), 256, gs, (const CopyArgs*)t);
         break;
       case REC_GEMM:
         e = launch_gemm_group((const GemmDesc*)t, S, r0.df, gs, nullptr);
