@@ -26,14 +26,14 @@
 // Work split: the columns of W, and with them the basis vectors that they become, are
 // spread over C CTAs of a cluster (range_ctas).  A step's O(n^2) column sweep is local;
 // between CTAs go the pivot candidates, the pivot column and the re-orthogonalisation's
-// partial sums (row slices summed over the CTAs in lane order, deterministic).  One CTA
+// partial sums (summed over the CTAs in a fixed order, deterministic).  One CTA
 // spends a step on ~10 n^2 FMAs at two FP64 operations per clock; with C of them a step
-// is bound by its three barriers and the latency of what is read between them.
+// is bound by its two or three barriers and the latency of what is read between them.
 //
 // Measured on GB300, a cold G of rank r with weights over 1e-12 (against one CTA of 512
 // threads sweeping all columns, the kernel of the sizes above 256): FP64 n = 32, r = 16
-// 110 us (360), n = 64, r = 32 274 us (987), n = 128, r = 64 0.84 ms (4.47); double-float
-// 79 us (124), 239 us (348), 0.71 ms (2.25).  FP64 runs on four warps instead of eight, with
+// 102 us (360), n = 64, r = 32 266 us (987), n = 128, r = 64 0.84 ms (4.47); double-float
+// 79 us (124), 227 us (348), 0.71 ms (2.25).  FP64 runs on four warps instead of eight, with
 // its comparisons off the FP64 pipe (n = 64 333 us and n = 128 0.94 ms on eight): what every
 // warp computes for itself held the pipes for ~6,000 of a step's ~20,000 cycles.
 //
@@ -59,6 +59,12 @@ struct RangeEps<df64> {
 };
 
 constexpr int RB_LOCAL = 48;  // columns of one CTA at most
+// Up to this many parts of rows, on up to eight CTAs, every CTA reads and sums all of them;
+// beyond, each sums a slice of the rows and hands it on (a barrier and a trip more): FP64 n = 32,
+// eight CTAs, 102 us against 110, n = 64 266 against 274; double-float n = 64, four CTAs, 227
+// against 239, but n = 128, eight CTAs, 757 against 707.
+constexpr int RB_ALL_PARTS = 512;
+constexpr int RB_ALL = 8;
 
 // CTAs that work on a problem of size n (a power of two).  One CTA needs no exchange (three
 // barriers and four reads across CTAs, ~5,000 cycles a step) and takes ~5 n^2 cycles for the
@@ -108,7 +114,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
   typedef Candidate<R> Cand;
   // (raw storage: double-float has a constructor)
   __shared__ __align__(16) unsigned char v_raw[FC_MAX_N * sizeof(cx<R>)];
-  __shared__ __align__(16) unsigned char y_raw[FC_MAX_N * sizeof(cx<R>)];
+  __shared__ __align__(16) unsigned char y_raw[2 * FC_MAX_N * sizeof(cx<R>)];
   __shared__ __align__(16) unsigned char z_raw[32 * sizeof(cx<R>)];
   __shared__ __align__(16) unsigned char c_raw[RB_LOCAL * sizeof(cx<R>)];
   __shared__ __align__(16) unsigned char part_raw[NW * sizeof(Cand)];
@@ -116,7 +122,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
   __shared__ __align__(16) unsigned char red_raw[NW * 2 * sizeof(R)];
   __shared__ __align__(16) unsigned char sums_raw[2 * sizeof(R)];
   cx<R>* const s_v = (cx<R>*)v_raw;      // the pivot column, then the new basis vector (a copy in every CTA)
-  cx<R>* const s_y = (cx<R>*)y_raw;      // our basis vectors' part of Q Q^dag v; read by the others
+  cx<R>* s_y = (cx<R>*)y_raw;            // our basis vectors' part of Q Q^dag v, two in turn; read by the others
   cx<R>* const s_z = (cx<R>*)z_raw;      // our slice of the projected column; read by the others
   cx<R>* const s_c = (cx<R>*)c_raw;      // q_i^dag v of our basis vectors
   Cand* const s_part = (Cand*)part_raw;  // per warp
@@ -149,6 +155,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
   };
 
   const int cpb = (n + ca - 1) / ca;  // columns (and rows of a slice) per CTA
+  const bool all_rows = ca <= RB_ALL && ca * n <= RB_ALL_PARTS;
   const int k0c = rank * cpb;
   const int ncl = max(0, min(n, k0c + cpb) - k0c);
   cx<R>* W = (cx<R>*)smem_raw;  // our columns, each contiguous
@@ -386,7 +393,27 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
           }
         }
         csync();
-        if (ca > 1) {
+        if (ca > 1 && all_rows) {
+          // v - the CTAs' parts, every row in every CTA, two lanes per row: one barrier and
+          // one trip between CTAs fewer than by slices, for ca n reads (the same sums in the
+          // same order)
+          for (int r0 = 0; r0 < n; r0 += NT / 2) {
+            if (r0 + warp * 16 >= n) break;  // no row for this warp
+            const int row = r0 + tid / 2, half = (tid & 1) * (ca / 2);
+            cx<R> y[RB_ALL / 2];
+#pragma unroll
+            for (int c = 0; c < RB_ALL / 2; c++)
+              y[c] = c < ca / 2 && row < n ? *on_cta(&s_y[row], half + c) : mk<R>(zero, zero);
+#pragma unroll
+            for (int o = 1; o < RB_ALL / 2; o <<= 1)
+#pragma unroll
+              for (int c = 0; c < RB_ALL / 2; c += 2 * o) y[c] = mk<R>(y[c].re + y[c + o].re, y[c].im + y[c + o].im);
+            y[0].re = y[0].re + sx(y[0].re, 1);
+            y[0].im = y[0].im + sx(y[0].im, 1);
+            if (row < n && !(tid & 1)) s_v[row] = csub_r(s_v[row], y[0]);
+          }
+          __syncthreads();
+        } else if (ca > 1) {
           // our slice of rows: v - the CTAs' parts, ca lanes per row
           for (int s0 = 0; s0 < ncl; s0 += NT / ca) {
             const int sr = s0 + tid / ca, sc = tid & (ca - 1), srow = k0c + sr;
@@ -403,6 +430,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
           for (int i = tid; i < n; i += NT) s_v[i] = *on_cta(&s_z[i % cpb], i / cpb);
           __syncthreads();
         }
+        s_y = (cx<R>*)y_raw + (s_y == (cx<R>*)y_raw ? FC_MAX_N : 0);
         const R prev = nrm2;
         {
           Acc<R> re, im;
