@@ -6,7 +6,7 @@
 // captured as a CUDA graph.  On this GPU one SM retires ~2 FP64 FMAs per clock, so what
 // counts is how evenly the products are spread over the SMs: a 32 x 32 x 16 block of
 // complex products takes one SM 16 us, a 16 x 16 x 16 block 4 us, an 8 x 8 x 16 block 1 us.
-// The kernel is persistent over a fixed grid (four CTAs per SM) and decides the
+// The kernel is persistent over a fixed grid (at most four CTAs per SM) and decides the
 // decomposition at run time from the actual sizes: output tiles of 16 x 16 or 8 x 8 (the
 // eight warps of a CTA take a quarter of the K chunk each), whichever finishes first with
 // its padding counted, and, with a workspace, a split of the K range into s parts while
@@ -349,9 +349,10 @@ cudaError_t launch_gemm(const GemmDesc& g, const int* d_dims, cudaStream_t s, do
   const int full = g.ws && g.grid > 0 ? g.grid : gemm_grid_default();
   const int grid = g.ws ? full : (int)std::min<long>(planned, full);
   gg.split_grid = full;
+  const int ctas = g.ctas > 0 ? std::min(grid, g.ctas) : grid;
   if (g.df64)
-    return launch_after(k_gemm<df64, false>, dim3(grid), G_THREADS, s, gg, d_dims, prof, nullptr);
-  return launch_after(k_gemm<double, false>, dim3(grid), G_THREADS, s, gg, d_dims, prof, nullptr);
+    return launch_after(k_gemm<df64, false>, dim3(ctas), G_THREADS, s, gg, d_dims, prof, nullptr);
+  return launch_after(k_gemm<double, false>, dim3(ctas), G_THREADS, s, gg, d_dims, prof, nullptr);
 }
 
 // The same GEMM of S states in one launch: grid (per-member CTAs, S).  Every member

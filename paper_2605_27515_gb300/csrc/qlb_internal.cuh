@@ -120,6 +120,7 @@ struct GemmDesc {
   int ksplit;
   void* ws;
   int grid;
+  int ctas;  // CTAs launched at most (0: as many as the decomposition is decided for)
   // 1: FP64 operands multiplied and summed in double-float (~48-bit significands) on
   // the FP32 pipes; the result is stored in FP64
   int df64;

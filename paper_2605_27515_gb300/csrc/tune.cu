@@ -1,5 +1,5 @@
 // Autotuner of the launch shapes of the step: the cap on the run-time K split of
-// the zip-up Gram GEMM G = M M^dag, whose (2z) x (2z) output makes few 32 x 32 tiles
+// the zip-up Gram GEMM G = M M^dag, whose (2z) x (2z) output makes few tiles
 // over a long K = d D (the work-distributed GEMM splits K until its fixed grid is
 // full; more parts mean more partial tiles to add).  For every bucket (rows m,
 // inner size K) the tuner times the GEMM with caps 1, 2, 4, 8, 16 with CUDA events
