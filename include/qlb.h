@@ -445,6 +445,18 @@ qlb_status qlb_zgemm_check(int device, int engine, int m, int n, int k, const do
 qlb_status qlb_eig_check(int device, int precision, int solver, int n, const double* G, double tol, int cap,
                          double* lam, double* V, int* k_out, double* ms);
 
+/* Failure check of a kernel whose CTAs wait for one another: runs it once on a seeded
+ * n x n matrix (1 <= n <= 256; the SVD on n x 4n) with the barrier of CTA `cta` (0..15)
+ * expecting an arrival that never comes, so that a bounded wait of a second runs out.
+ *   kernel     0 the step's truncation solve, in its factorisation; 1 the same, in its
+ *              exchanges of columns; 2 the zip-up range basis; 3 the operator builder's
+ *              SVD (FP64 whatever the precision)
+ *   precision  QLB_PREC_F64 or QLB_PREC_MIXED
+ * QLB_ETIMEOUT when the wait ran out and every CTA left, QLB_OK when fewer than cta + 1
+ * CTAs work on this size (nothing waits for the missing arrival).  The device stays
+ * usable.  Takes two or three seconds. */
+qlb_status qlb_lost_wait_check(int device, int kernel, int precision, int n, int cta);
+
 #ifdef __cplusplus
 }
 #endif

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <random>
 #include <string>
 
 #include "step.cuh"
@@ -1009,8 +1010,9 @@ QLB_API qlb_status qlb_tc_zgemm(int device, int m, int n, int k, const double* A
 
 // ------------------------------------------------------------------ truncation-solver check
 
-QLB_API qlb_status qlb_eig_check(int device, int precision, int solver, int n, const double* G, double tol, int cap,
-                                 double* lam, double* V, int* k_out, double* ms) {
+// stall: EigDesc::stall (0: none)
+static qlb_status eig_check(int device, int precision, int solver, int n, const double* G, double tol, int cap,
+                            double* lam, double* V, int* k_out, double* ms, int stall) {
   CHECK_ARG(G && lam && V && k_out && ms, "null argument");
   CHECK_ARG(n >= 1 && n <= 512, "n must be in [1, 512]");
   CHECK_ARG(precision == QLB_PREC_F64 || precision == QLB_PREC_MIXED, "precision must be F64 or MIXED");
@@ -1076,11 +1078,12 @@ QLB_API qlb_status qlb_eig_check(int device, int precision, int solver, int n, c
   e.gap = 1e-10;
   e.max_sweeps = 40;
   e.err = dErr;
+  e.stall = stall;
   if (solver != 5) e.lam = dLam;
   const bool mixed = precision == QLB_PREC_MIXED;
   cudaError_t r = cudaSuccess;
   float t = 0.f;
-  for (int rep = 0; rep < 2 && r == cudaSuccess; rep++) {
+  for (int rep = 0; rep < (stall ? 1 : 2) && r == cudaSuccess; rep++) {
     cudaMemcpy(dG, dG0, sizeof(zd) * nn, cudaMemcpyDeviceToDevice);
     cudaMemset(dDims, 0, sizeof(int) * 4);
     cudaMemset(dErr, 0, sizeof(int));
@@ -1105,6 +1108,10 @@ QLB_API qlb_status qlb_eig_check(int device, int precision, int solver, int n, c
   }
   *k_out = gated ? -1 : k;
   *ms = t;
+  if (herr & 4) {
+    set_error("qlb_eig_check: a bounded wait between the solve's CTAs gave up");
+    return QLB_ETIMEOUT;
+  }
   if (herr & 2) {
     set_error("qlb_eig_check: non-finite values in the solve");
     return QLB_ENONFINITE;
@@ -1114,6 +1121,72 @@ QLB_API qlb_status qlb_eig_check(int device, int precision, int solver, int n, c
     return QLB_ENOTCONV;
   }
   return QLB_OK;
+}
+
+QLB_API qlb_status qlb_eig_check(int device, int precision, int solver, int n, const double* G, double tol, int cap,
+                                 double* lam, double* V, int* k_out, double* ms) {
+  return eig_check(device, precision, solver, n, G, tol, cap, lam, V, k_out, ms, 0);
+}
+
+// ------------------------------------------------------------------ lost-wait check
+
+// The operator SVD of the n x 4n matrix M in one launch, with CTA `cta` stalled.
+static qlb_status osj_lost_wait(int device, int n, const std::vector<double>& M, int cta) {
+  QLB_CUDA_TRY(cudaSetDevice(device));
+  init_kernel_attributes();
+  const size_t nn = (size_t)n * n;
+  zd* buf = nullptr;  // X, T, U, R, then the status and the kept count
+  if (cudaMalloc(&buf, sizeof(zd) * (10 * nn + 1)) != cudaSuccess) {
+    cudaGetLastError();
+    set_error("qlb_lost_wait_check: device allocation failed");
+    return QLB_ENOMEM;
+  }
+  int* d_out = (int*)(buf + 10 * nn);
+  const OsjOut out{1e-12, 1e-10, 0, 0, 0, 0, buf + 5 * nn, buf + 6 * nn, d_out + 1, cta + 1};
+  int h = 0;
+  cudaError_t e = cudaMemcpy(buf, M.data(), sizeof(zd) * 4 * nn, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_osj(buf, n, 4 * n, buf + 4 * nn, 60, d_out, out, 0);
+  if (e == cudaSuccess) e = cudaMemcpy(&h, d_out, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(buf);
+  QLB_CUDA_TRY(e);
+  if (h == -2) {
+    set_error("qlb_lost_wait_check: a bounded wait between the SVD's CTAs gave up");
+    return QLB_ETIMEOUT;
+  }
+  return h > 0 ? QLB_OK : QLB_ENOTCONV;
+}
+
+QLB_API qlb_status qlb_lost_wait_check(int device, int kernel, int precision, int n, int cta) {
+  CHECK_ARG(kernel >= 0 && kernel <= 3, "unknown kernel");
+  CHECK_ARG(n >= 1 && n <= 256, "n must be in [1, 256]");
+  CHECK_ARG(cta >= 0 && cta < 16, "cta must be in [0, 16)");
+  int ndev = 0;
+  if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) {
+    cudaGetLastError();
+    set_error("qlb_lost_wait_check: no such CUDA device");
+    return QLB_EDEVICE;
+  }
+  std::vector<double> M(8 * (size_t)n * n);
+  std::mt19937_64 rng(n);
+  std::normal_distribution<double> nd;
+  for (double& x : M) x = nd(rng);
+  if (kernel == 3) return osj_lost_wait(device, n, M, cta);
+  std::vector<double> G(2 * (size_t)n * n), V(G.size()), lam(n);  // M M^dag of the first n columns
+  for (int i = 0; i < n; i++)
+    for (int j = 0; j < n; j++) {
+      double re = 0, im = 0;
+      for (int k = 0; k < n; k++) {
+        const double *a = &M[2 * ((size_t)i * n + k)], *b = &M[2 * ((size_t)j * n + k)];
+        re += a[0] * b[0] + a[1] * b[1];
+        im += a[1] * b[0] - a[0] * b[1];
+      }
+      G[2 * ((size_t)i * n + j)] = re;
+      G[2 * ((size_t)i * n + j) + 1] = im;
+    }
+  int k = 0;
+  double ms = 0;
+  return eig_check(device, precision, kernel == 2 ? 5 : 0, n, G.data(), 1e-12, n, lam.data(), V.data(), &k, &ms,
+                   kernel == 1 ? -cta - 1 : cta + 1);
 }
 
 // ------------------------------------------------------------------ GEMM engine check

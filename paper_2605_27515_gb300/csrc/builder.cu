@@ -315,7 +315,7 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
     return st;
   zd* T = (zd*)bt.p;
   int* d_cnt = (int*)bc.p;  // sweeps or rotations, then the kept count
-  const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, tall, (zd*)bu.p, (zd*)br.p, d_cnt + 1};
+  const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, tall, (zd*)bu.p, (zd*)br.p, d_cnt + 1, 0};
   int h[2] = {0, 0};
   if (osj_serves(m, n)) {
     QLB_CUDA_TRY(launch_osj(X, m, n, T, max_sweeps, d_cnt, out, s));
@@ -345,6 +345,10 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   if (e != cudaSuccess) {
     set_error(std::string("svd finish: ") + cudaGetErrorString(e));
     return QLB_EDEVICE;
+  }
+  if (h[0] == -2) {
+    set_error("a bounded wait of the one-sided Jacobi SVD gave up");
+    return QLB_ETIMEOUT;
   }
   if (h[0] <= 0) {
     set_error("one-sided Jacobi SVD did not converge");

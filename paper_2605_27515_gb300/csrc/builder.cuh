@@ -73,6 +73,7 @@ struct OsjOut {
   int cap, u_scale, r_unscale, tall;
   zd *U, *Rr;
   int* k_out;
+  int stall;  // failure test: 1 + the CTA whose barrier expects an arrival that never comes
 };
 bool osj_serves(int m, int n);
 // all sweeps on the rows of X (m x n; may be overwritten, like T, m x m) and the factors

@@ -86,22 +86,55 @@ __device__ __forceinline__ bool bounded_wait(const unsigned long long* bar, unsi
 // Barrier over the CTAs that work on the problem, in two halves: every CTA's mbarrier
 // counts one arrival of each of them.  Unlike the hardware's cluster barrier it leaves out
 // the CTAs that have nothing to do, and its waits are bounded.
+//
+// A wait that gives up is lost for the whole CTA (`lost` is the same in every thread): the
+// CTA takes part in no further phase and goes to leave(), where the others meet it, as
+// their next wait gives up too.  The vote costs a block barrier a phase (~1 % of a step).
 struct ClusterBarrier {
   const unsigned long long* bar;
+  int* gave_up;  // of this CTA; set by any CTA that lost a wait
   int ca;
   unsigned phase;
   bool lost;
-  __device__ __forceinline__ void arrive() {
-    __syncthreads();
+  // what one thread's bounded wait came to, for all threads; a block barrier
+  __device__ __forceinline__ bool agree(bool ok) {
+    lost = __syncthreads_or(!ok) != 0;
+    return !lost;
+  }
+  // behind a block barrier
+  __device__ __forceinline__ void post() {
     if ((int)threadIdx.x < ca) {
       unsigned rb;
       asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_addr(bar)), "r"((int)threadIdx.x));
       asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rb) : "memory");
     }
   }
-  __device__ __forceinline__ void wait() {
-    if (!lost && !bounded_wait(bar, phase & 1)) lost = true;
-    phase++;
+  __device__ __forceinline__ void arrive() {
+    __syncthreads();
+    post();
+  }
+  __device__ __forceinline__ bool wait() { return agree(bounded_wait(bar, phase++ & 1)); }
+  __device__ __forceinline__ bool sync() {
+    if (ca == 1) {
+      __syncthreads();
+      return true;
+    }
+    arrive();
+    return wait();
+  }
+  // The way out of every CTA that works on the problem, lost or not: none of them touches
+  // another one's shared memory any more.  True when any lost a wait (the same in all).  The
+  // hardware's barrier waits for the CTAs that have not exited; each reaches it, as the
+  // waits before are bounded and a lost CTA skips the rest.
+  __device__ __forceinline__ bool leave() {
+    if (ca == 1) {
+      __syncthreads();
+      return false;
+    }
+    if (lost && (int)threadIdx.x < ca) *on_cta(gave_up, (int)threadIdx.x) = 1;
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    return *(volatile int*)gave_up != 0;
   }
 };
 

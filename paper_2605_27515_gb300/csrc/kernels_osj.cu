@@ -152,7 +152,7 @@ __host__ __device__ inline size_t osj_head_bytes(int m, int g) {
 }
 __host__ __device__ inline int osj_ld(int n, int m, int ca) { return ((n + ca - 1) / ca + (m + ca - 1) / ca) | 1; }
 
-// sweeps_out: the sweeps run, or -1 when max_sweeps did not do
+// sweeps_out: the sweeps run, -1 when max_sweeps did not do, -2 when a bounded wait gave up
 __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, int max_sweeps, int* sweeps_out,
                                                    int resident, OsjOut out) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
   __shared__ double s_f2[OSJ_NW];
   __shared__ double s_mine;  // our part of ||X||_F^2; read by the others
   __shared__ unsigned s_mc, s_ms;
-  __shared__ int s_k;
+  __shared__ int s_k, s_gave_up;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ca = (int)gridDim.x, rank = (int)cta_rank_in_cluster();
   const int wn = (n + ca - 1) / ca, wm = (m + ca - 1) / ca;
@@ -172,22 +172,17 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
   int* const perm = (int*)(ws + m);
 
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_cbar)), "r"(ca) : "memory");
+    s_gave_up = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_cbar)),
+                 "r"(ca + (out.stall == rank + 1))
+                 : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   // once, with every CTA of the cluster: the barrier above is set up
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  ClusterBarrier cb{&s_cbar, ca, 0u, false};
-  auto csync = [&]() {
-    if (ca == 1) {
-      __syncthreads();
-    } else {
-      cb.arrive();
-      cb.wait();
-    }
-  };
+  ClusterBarrier cb{&s_cbar, &s_gave_up, ca, 0u, false};
 
   OsjSlice c;
   c.j0 = min(n, rank * wn);
@@ -222,9 +217,9 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
     s_mine = s;
     s_mc = s_ms = 0u;
   }
-  csync();
+  cb.sync();
   f2 = 0.0;
-  for (int r = 0; r < ca; r++) f2 += *on_cta(&s_mine, r);
+  for (int r = 0; r < ca && !cb.lost; r++) f2 += *on_cta(&s_mine, r);
 
   // A pair is rotated only when |x_p . x_q| exceeds both ~sqrt(n) eps |x_p| |x_q| (a length-n
   // dot product carries that much rounding) and 1e-31 ||X||_F^2: without the absolute floor, the
@@ -236,7 +231,7 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
   const int sub = gl / 32, base = lane & ~(GW - 1);
   int sweep = 0;
   bool converged = !usable || m <= 1;
-  for (int par = 0; !converged && sweep < max_sweeps; sweep++) {
+  for (int par = 0; !converged && !cb.lost && sweep < max_sweeps; sweep++) {
     float mc = 0.f, ms = 0.f;
     for (int round = 0; round < np - 1; round++, par ^= 1) {
       PairSums* const mine = part + par * pairs * nsub;
@@ -268,7 +263,7 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
         for (int o = 4; o < GW; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (k < pairs && (gl & 31) < 4) mine[k * nsub + sub].v[lane & 3] = v;
       }
-      csync();
+      if (!cb.sync()) break;
       for (int k0 = 0; k0 < pairs; k0 += ng) {
         if (k0 + (warp * 32) / G >= pairs) break;
         const int k = k0 + gid;
@@ -343,6 +338,7 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
       }
       __syncthreads();
     }
+    if (cb.lost) break;
     mc = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mc)));
     ms = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ms)));
     if (lane == 0 && mc > 0.f) {
@@ -361,23 +357,23 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
   }
 
   // row norms, truncation rule (alike in every CTA), our columns of the factors
-  for (int p = warp; p < m; p += OSJ_NW) {
-    double acc = 0;
-    for (int j = lane; j < c.nl; j += 32) acc += cabs2(c.x[p * c.ldx + j]);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) ws[p] = acc;  // read by the others
+  if (!cb.lost) {
+    for (int p = warp; p < m; p += OSJ_NW) {
+      double acc = 0;
+      for (int j = lane; j < c.nl; j += 32) acc += cabs2(c.x[p * c.ldx + j]);
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) ws[p] = acc;  // read by the others
+    }
+    if (cb.sync())
+      for (int p = tid; p < m; p += OSJ_NT) {
+        double acc = 0;
+        for (int r = 0; r < ca; r++) acc += *on_cta(&ws[p], r);
+        w[p] = acc;
+      }
   }
-  csync();
-  for (int p = tid; p < m; p += OSJ_NT) {
-    double acc = 0;
-    for (int r = 0; r < ca; r++) acc += *on_cta(&ws[p], r);
-    w[p] = acc;
-  }
-  // the last access to another CTA's shared memory
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  if (cb.lost) converged = false;
-  if (rank == 0 && tid == 0) *sweeps_out = converged ? max(1, sweep) : -1;
+  const bool gave_up = cb.leave();
+  if (rank == 0 && tid == 0) *sweeps_out = gave_up ? -2 : converged ? max(1, sweep) : -1;
+  if (gave_up) return;  // no factors
   const int k = osj_rule(w, ws, perm, &s_k, m, out.tol, out.cap, out.gap);
   if (rank == 0 && tid == 0) *out.k_out = k;
   osj_write(c, w, ws, perm, m, n, k, out);

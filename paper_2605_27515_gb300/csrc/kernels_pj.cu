@@ -87,6 +87,7 @@ struct __align__(16) FactorSmem {
   unsigned long long cbar;           // every working CTA has arrived
   unsigned key[3];                   // our best pivot candidate
   int bad;
+  int gave_up;                       // a CTA lost a wait
 };
 
 struct Factor {
@@ -96,14 +97,18 @@ struct Factor {
   double down;   // the power of two that undoes the scale of L L^dag
 };
 
-// Sets up fs and the barrier over the ca CTAs that work on the problem; false for the
-// others, which leave.  Every thread of every CTA of the cluster calls it.
-__device__ __forceinline__ bool factor_begin(FactorSmem& fs, unsigned long long* more, int ca, int rank) {
+// Sets up fs, the barrier over the ca CTAs that work on the problem and the one of the
+// exchanges (`more`); false for the other CTAs, which leave.  Every thread of every CTA of the
+// cluster calls it.
+__device__ __forceinline__ bool factor_begin(FactorSmem& fs, unsigned long long* more, int ca, int rank, int stall) {
   if (threadIdx.x == 0) {
     fs.bad = 0;
+    fs.gave_up = 0;
     fs.key[0] = fs.key[1] = fs.key[2] = 0u;
-    if (more) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(more)) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&fs.cbar)), "r"(ca) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(more)), "r"(1 + (stall == -rank - 1))
+                 : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&fs.cbar)), "r"(ca + (stall == rank + 1))
+                 : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -117,7 +122,8 @@ __device__ __forceinline__ bool factor_begin(FactorSmem& fs, unsigned long long*
 // decomposition of a semi-definite matrix", 1990).  CTA `rank` of ca works on rows
 // [rank * rpb, (rank + 1) * rpb): Gl and Ll are theirs, row-major with stride n, G scaled by
 // a power of two to a trace in [1, 2).  A pivot is taken while its residual stands above
-// eps times its diagonal entry of G.  One barrier per pivot; ends with one.
+// eps times its diagonal entry of G.  One barrier per pivot; ends with one.  When a wait is
+// lost (cb.lost) there is no factor.
 template <typename R>
 __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd* G, int n, int ca, int rank,
                                    cx<R>* Gl, cx<R>* Ll) {
@@ -127,14 +133,6 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
   cx<R>* const s_row = (cx<R>*)fs.row;
   R* const s_d = (R*)fs.d;
   R* const s_floor = (R*)fs.floor;
-  auto csync = [&]() {
-    if (ca == 1) {
-      __syncthreads();
-    } else {
-      cb.arrive();
-      cb.wait();
-    }
-  };
   const int rpb = (n + ca - 1) / ca;
   const int r0 = rank * rpb;
   const int nl = max(0, min(n, r0 + rpb) - r0);
@@ -190,7 +188,7 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
     key = __reduce_max_sync(0xffffffffu, key);
     if (lane == 0 && key) atomicMax(&fs.key[0], key);
   }
-  csync();
+  if (!cb.sync()) return out;
   for (int c = 0; c < ca; c++) out.bad = out.bad || *on_cta(&fs.bad, c) != 0;
   int r = 0;
   if (!out.bad && tr_ok) {
@@ -249,10 +247,10 @@ __device__ Factor pivoted_cholesky(FactorSmem& fs, ClusterBarrier& cb, const zd*
       }
       best = __reduce_max_sync(0xffffffffu, best);
       if (lane == 0 && best) atomicMax(&fs.key[set], best);
-      csync();
+      if (!cb.sync()) return out;
     }
   }
-  csync();  // nobody reads another CTA's candidates any more
+  cb.sync();  // nobody reads another CTA's candidates any more
   out.r = r;
   return out;
 }
@@ -300,16 +298,8 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
   __shared__ int s_bad, s_k;
   __shared__ __align__(8) unsigned long long s_bar;  // the two blocks of an exchange have arrived
 
-  if (!factor_begin(fs, &s_bar, ca, rank)) return;
-  ClusterBarrier cb{&fs.cbar, ca, 0u, false};
-  auto csync = [&]() {
-    if (ca == 1) {
-      __syncthreads();
-    } else {
-      cb.arrive();
-      cb.wait();
-    }
-  };
+  if (!factor_begin(fs, &s_bar, ca, rank, e.stall)) return;
+  ClusterBarrier cb{&fs.cbar, &fs.gave_up, ca, 0u, false};
 
   // ---- 1. pivoted Cholesky
   const int rpb = (n + ca - 1) / ca;
@@ -317,7 +307,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
   cx<R>* buf1 = buf0 + pj_region(n, ca);
   cx<R>* Ll = buf1;
   const Factor f = pivoted_cholesky<R>(fs, cb, (const zd*)e.G, n, ca, rank, buf0, Ll);
-  const int r = f.r;
+  int r = f.r;
   const bool any_bad = f.bad;
   const double tr = f.tr, down = f.down;
 
@@ -327,7 +317,10 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
   const int ld = n + 1;  // a column and its squared norm
   cx<R>* cur = buf0;
   cx<R>* nxt = buf1;
-  for (int x = tid; x < nc * n; x += NT) {
+  // blocks may be sent to us from the barrier below on
+  const bool exchanging = ca > 1 && !cb.lost;
+  bool armed = false;  // s_bar expects this turn's blocks
+  for (int x = tid; x < nc * n && !cb.lost; x += NT) {
     const int i = x / nc, s = x - i * nc;
     const int t = s < b ? rank * b + s : (ca + rank) * b + (s - b);
     const int o = i / rpb;
@@ -335,7 +328,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
     if (t < r) v = on_cta(Ll, o)[(long)(i - o * rpb) * n + t];
     cur[(long)s * ld + i] = v;
   }
-  csync();  // every CTA has read the factor before its rows become the next column buffer
+  if (!cb.lost) cb.sync();  // every CTA has read the factor before its rows become the next column buffer
 
   // lanes per pair: enough warps to fill the SM's four partitions, as in the factorisation
   const int want = std::is_same<R, double>::value ? 4 : 8;
@@ -358,9 +351,9 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
   int sweep = 0;
   long total_rot = 0;
   int turn = 0;
-  bool converged = false, measure = false, pending = false, lost = false;
+  bool converged = false, measure = false, pending = false;
   double off2 = 0.0;
-  for (;; sweep++) {
+  for (; !cb.lost; sweep++) {
     int nrot = 0;
     float mc = 0.f, ms = 0.f;
     double off_l = 0.0;
@@ -462,8 +455,10 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
         // exchange at n = 64 over 8 CTAs (10,200 at n = 128 over 16), remote loads 5,300
         // (6,500), most of it their acknowledgement.
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (pending) cb.wait();  // every CTA's next buffer has been sent on
+        if (!pending)
+          __syncthreads();
+        else if (!cb.wait())  // every CTA's next buffer has been sent on
+          break;
         if (tid == 0) {
           const unsigned bytes = (unsigned)(b * ld * sizeof(cx<R>));
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_bar)),
@@ -474,11 +469,13 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
           send_block(tc, nxt + (long)ts * ld, cur, bytes, &s_bar);
           send_block(rank == 0 ? 1 : rank - 1, nxt + (rank == 0 ? 0 : (long)b * ld), cur + (long)b * ld, bytes, &s_bar);
         }
-        if (!lost && !bounded_wait(&s_bar, turn & 1)) lost = true;  // reported below; no further wait
+        armed = true;
+        if (!cb.agree(bounded_wait(&s_bar, turn & 1))) break;
+        armed = false;
         turn++;
-        cb.arrive();  // our two blocks are here, so their senders' buffers are free
+        cb.post();  // our two blocks are here, so their senders' buffers are free
         pending = o < 2 * ca - 2;
-        if (!pending) cb.wait();  // the sweep's rotations of every CTA are there
+        if (!pending && !cb.wait()) break;  // the sweep's rotations of every CTA are there
         cx<R>* t = cur;
         cur = nxt;
         nxt = t;
@@ -486,10 +483,11 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
         __syncthreads();
       }
     }
+    if (cb.lost) break;
     if (measure) {
       for (int s = 16; s > 0; s >>= 1) off_l += __shfl_xor_sync(0xffffffffu, off_l, s);
       if (lane == 0) s_off[warp] = off_l;
-      csync();
+      if (!cb.sync()) break;
       for (int c = 0; c < ca * NW; c++) off2 += *on_cta(&s_off[c % NW], c / NW);
       break;
     }
@@ -517,20 +515,33 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
     if (sweep + 1 >= e.max_sweeps) measure = true;  // one pass that only sums the couplings left
   }
 
-  if ((lost || cb.lost) && e.err) atomicOr(e.err, 4);
-
   // ---- 3. weights, kept count, vectors
   const int ns = nc * ca;
-  for (int k0 = 0; k0 < nc; k0 += npg) {
-    if (k0 + (warp * 32) / LP >= nc) break;
-    const int k = k0 + pg;
-    const R na = norm2(k);
-    if (k < nc && pl == 0) s_own[k] = (double)na * down;
+  if (!cb.lost) {
+    for (int k0 = 0; k0 < nc; k0 += npg) {
+      if (k0 + (warp * 32) / LP >= nc) break;
+      const int k = k0 + pg;
+      const R na = norm2(k);
+      if (k < nc && pl == 0) s_own[k] = (double)na * down;
+    }
+    if (cb.sync())
+      for (int i = tid; i < ns; i += NT) s_lam[i] = *on_cta(&s_own[i % nc], i / nc);
   }
-  csync();
-  for (int i = tid; i < ns; i += NT) s_lam[i] = *on_cta(&s_own[i % nc], i / nc);
-  csync();  // the last access to another CTA's shared memory
+  // blocks that the others have sent us by now land before anyone leaves: a sender is at
+  // most one turn ahead of us, and waits in leave() meanwhile
+  if (cb.lost && exchanging) {
+    if (!armed && tid == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_bar)),
+                   "r"((unsigned)(2 * b * ld * sizeof(cx<R>)))
+                   : "memory");
+    bounded_wait(&s_bar, turn & 1);
+  }
+  const bool gave_up = cb.leave();
   let_next_start();
+  if (gave_up) {  // one unit vector and the flag
+    r = 0;
+    for (int i = tid; i < ns; i += NT) s_lam[i] = 0.0;
+  }
   if (tid == 0) s_bad = any_bad ? 1 : 0;
   __syncthreads();
   for (int i = tid; i < ns; i += NT) {
@@ -562,7 +573,8 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
         if (dr > *e.disc_stat) *e.disc_stat = dr;
       }
       if (e.err) {
-        if (!converged && !s_bad && !(::sqrt(off2) * down <= (double)n * FcEps<R>::v * tr)) atomicOr(e.err, 1);
+        if (gave_up) atomicOr(e.err, 4);
+        if (!gave_up && !converged && !s_bad && !(::sqrt(off2) * down <= (double)n * FcEps<R>::v * tr)) atomicOr(e.err, 1);
         if (s_bad) atomicOr(e.err, 2);
       }
       if (e.solver_stats) {
@@ -570,7 +582,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
         atomicAdd(e.solver_stats + 1, (double)(converged ? sweep + 1 : e.max_sweeps));
         atomicAdd(e.solver_stats + 2, (double)n);
         atomicAdd(e.solver_stats + 3, (double)k);
-        if (!converged) atomicAdd(e.solver_stats + 4, 1.0);
+        if (!converged && !gave_up) atomicAdd(e.solver_stats + 4, 1.0);
         if (ca > 1) atomicAdd(e.solver_stats + 5, 1.0);  // a multi-SM solve
         atomicMax((unsigned long long*)(e.solver_stats + 6), (unsigned long long)__double_as_longlong((double)n));
       }
@@ -586,7 +598,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_pj(EigDesc e, int* d, do
     for (int i = tid; i < n; i += NT) e.lam[i] = r > 0 && i < ns ? s_w[i] : 0.0;
   zd* out = (zd*)e.out;
   if (e.out_mode != 0 && e.out_mode != 1) return;
-  if (r == 0) {  // nothing above rounding (or non-finite entries): one unit vector
+  if (r == 0) {  // nothing above rounding (or non-finite entries, a lost wait): one unit vector
     if (rank == 0)
       for (int i = tid; i < n; i += NT) out[i] = mk<double>(i == 0 ? 1.0 : 0.0, 0.0);
     return;

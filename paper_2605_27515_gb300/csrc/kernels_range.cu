@@ -132,11 +132,14 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
   __shared__ unsigned char s_done[RB_LOCAL];
   __shared__ short s_slot[RB_LOCAL], s_idx[RB_LOCAL];  // our basis vectors: column slot, index j
   __shared__ unsigned long long s_cbar;
-  __shared__ int s_bad;
+  __shared__ int s_bad, s_gave_up;
 
   if (tid == 0) {
     s_bad = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_cbar)), "r"(ca) : "memory");
+    s_gave_up = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_cbar)),
+                 "r"(ca + (e.stall == rank + 1))
+                 : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -144,15 +147,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
   if (rank >= ca) return;
-  ClusterBarrier cb{&s_cbar, ca, 0u, false};
-  auto csync = [&]() {
-    if (ca == 1) {
-      __syncthreads();
-    } else {
-      cb.arrive();
-      cb.wait();
-    }
-  };
+  ClusterBarrier cb{&s_cbar, &s_gave_up, ca, 0u, false};
 
   const int cpb = (n + ca - 1) / ca;  // columns (and rows of a slice) per CTA
   const bool all_rows = ca <= RB_ALL && ca * n <= RB_ALL_PARTS;
@@ -300,9 +295,9 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
     s_sums[1] = tr;
   }
   column_sweep(nullptr, 0);
-  csync();
+  cb.sync();
   bool any_bad = s_bad != 0;
-  if (ca > 1) {
+  if (ca > 1 && !cb.lost) {
     fr = zero;
     tr = zero;
     any_bad = false;
@@ -316,11 +311,11 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
   const R thr_w = R(e.tol) * tr;
   const R floor2 = R(RangeEps<R>::v * RangeEps<R>::v) * fr;
   const R quarter = from_f(R(), 0.25f);
-  const bool usable = !any_bad && fr > zero;
+  bool usable = !any_bad && fr > zero;
   double flops = 0.0;  // thread 0 only
   int j = 0, jl = 0;   // basis vectors, ours of them
   bool fallback = false;
-  if (usable) {
+  if (usable && !cb.lost) {
     for (int par = 0;; j++, par ^= 1) {
       // the candidates, reduced alike in every warp of every CTA
       Cand c;
@@ -392,7 +387,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
               s_y[row] = y;
           }
         }
-        csync();
+        if (!cb.sync()) break;
         if (ca > 1 && all_rows) {
           // v - the CTAs' parts, every row in every CTA, two lanes per row: one barrier and
           // one trip between CTAs fewer than by slices, for ca n reads (the same sums in the
@@ -426,7 +421,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
             }
             if (sr < ncl && sc == 0) s_z[sr] = csub_r(s_v[srow], y);
           }
-          csync();
+          if (!cb.sync()) break;
           for (int i = tid; i < n; i += NT) s_v[i] = *on_cta(&s_z[i % cpb], i / cpb);
           __syncthreads();
         }
@@ -446,10 +441,11 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
         if (tid == 0) flops += 16.0 * n * j;
         if (le_nn(quarter * prev, nrm2)) break;
       }
+      if (cb.lost) break;
       // the pivot's true residual is at the rounding level: what the tracked norms still
       // show is rounding of earlier projections, and the range is complete
       if (j >= 1 && le_nn(nrm2, floor2)) break;
-      if (j == 0) csync();  // every CTA has read the column that becomes q_0
+      if (j == 0 && !cb.sync()) break;  // every CTA has read the column that becomes q_0
       {
         const R inv = rsqrt_r(nrm2);
         for (int i = tid; i < n; i += NT) {
@@ -469,14 +465,15 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
       __syncthreads();
       column_sweep(s_v, par ^ 1);
       if (tid == 0) flops += 20.0 * n * (n - j - 1);
-      csync();
+      if (!cb.sync()) break;
     }
   }
-  csync();  // nobody reads another CTA's shared memory any more
+  const bool gave_up = cb.leave();
   let_next_start();
+  if (gave_up) usable = fallback = false;  // one unit vector and the flag
   const int r = usable ? j : 1;
   if (rank == 0 && tid == 0) {
-    if (cb.lost && e.err) atomicOr(e.err, 4);
+    if (gave_up && e.err) atomicOr(e.err, 4);
     if (e.gate) *e.gate = fallback ? 1 : 0;
     if (!fallback) {
       d[e.dim_out] = r;
@@ -506,7 +503,7 @@ __global__ void __launch_bounds__(ClThreads<R>::v, 1) k_range(EigDesc e, int* d,
     else if (e.out_mode == 1)
       out[(long)jj * n + i] = mk<double>(re, -im);
   };
-  if (!usable) {  // G = 0 or non-finite entries: one unit vector
+  if (!usable) {  // G = 0, non-finite entries or a lost wait: one unit vector
     if (rank == 0)
       for (int i = tid; i < n; i += NT) put(i, 0, i == 0 ? 1.0 : 0.0, 0.0);
     return;

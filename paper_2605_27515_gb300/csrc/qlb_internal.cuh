@@ -150,6 +150,8 @@ struct EigDesc {
   double gap;        // degeneracy gap
   int max_sweeps;
   int two_sided;     // 1: two-sided Jacobi at every size (the solve of every zip-up bond)
+  int stall;         // failure test: 1 + the CTA of a cluster kernel whose barrier expects an
+                     // arrival that never comes (-1 - the CTA: the barrier of k_pj's exchanges)
   double* kept_weight;  // optional: sum of kept eigenvalues
   double* total_weight; // optional: sum of all eigenvalues
   double* disc_stat;    // optional: running max of discarded relative weight

@@ -83,6 +83,7 @@ _SIGS = {
     "qlb_eig_check": (_st, [C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_double), C.c_double, C.c_int,
                             C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_int),
                             C.POINTER(C.c_double)]),
+    "qlb_lost_wait_check": (_st, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int]),
     "qlb_system_create": (_st, [_vp, C.c_int, C.POINTER(C.c_int), C.POINTER(_vp)]),
     "qlb_system_destroy": (None, [_vp]),
     "qlb_op_build": (_st, [_vp, C.POINTER(qlb_term), C.c_int, C.c_double, C.c_int, C.POINTER(_vp)]),
@@ -488,6 +489,14 @@ def qlb_eig_check(device: int, precision: int, solver: int, G, tol: float = 0.0,
                                 C.byref(ms)))
     kk = k.value
     return lam, (V[:n * kk].reshape(n, kk) if kk > 0 else None), kk, ms.value
+
+
+WAIT_FACTOR, WAIT_EXCHANGE, WAIT_RANGE, WAIT_SVD = range(4)
+
+
+def qlb_lost_wait_check(device: int, kernel: int, precision: int, n: int, cta: int):
+    """One cluster kernel with a barrier of CTA `cta` that never completes; raises ETIMEOUT."""
+    _check(load().qlb_lost_wait_check(int(device), int(kernel), int(precision), int(n), int(cta)))
 
 
 class Group:
