@@ -445,6 +445,12 @@ qlb_status qlb_zgemm_check(int device, int engine, int m, int n, int k, const do
 qlb_status qlb_eig_check(int device, int precision, int solver, int n, const double* G, double tol, int cap,
                          double* lam, double* V, int* k_out, double* ms);
 
+/* Failure injection on the host: sets the error flags that the kernels of a state's next
+ * call may set, so that the call reports them: 1 a solve hit its sweep limit
+ * (QLB_ENOTCONV), 2 non-finite values (QLB_ENONFINITE), 4 a bounded wait gave up
+ * (QLB_ETIMEOUT); of several the last named counts.  The call's work is done as usual. */
+qlb_status qlb_inject_flags(qlb_state* st, int flags);
+
 /* Failure check of a kernel whose CTAs wait for one another: runs it once on a seeded
  * n x n matrix (1 <= n <= 256; the SVD on n x 4n) with the barrier of CTA `cta` (0..15)
  * expecting an arrival that never comes, so that a bounded wait of a second runs out.

@@ -660,6 +660,14 @@ QLB_API void qlb_state_destroy(qlb_state* st) {
   delete st;
 }
 
+QLB_API qlb_status qlb_inject_flags(qlb_state* st, int flags) {
+  CHECK_ARG(st, "null state");
+  CHECK_ARG(flags >= 0 && flags <= 7, "unknown flags");
+  QLB_CUDA_TRY(cudaStreamSynchronize(st->stream));
+  QLB_CUDA_TRY(cudaMemcpy(st->d_err, &flags, sizeof(int), cudaMemcpyHostToDevice));
+  return QLB_OK;
+}
+
 QLB_API qlb_status qlb_truncate(qlb_state* st, double tol, int chi_max, int chi_mu_max) {
   CHECK_ARG(st, "null state");
   CHECK_ARG(tol < 1, "tol must be < 1");

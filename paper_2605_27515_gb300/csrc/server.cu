@@ -236,10 +236,8 @@ void qlb_server::finish(std::shared_ptr<Job>& j, bool ok) {
     int err = 0;
     cudaMemcpy(&err, j->st->d_err, sizeof(int), cudaMemcpyDeviceToHost);
     if (err) {
-      j->status = (err & 4) ? QLB_ETIMEOUT : (err & 2) ? QLB_ENONFINITE : QLB_ENOTCONV;
-      j->error = (err & 4)   ? "a bounded wait of the tensor-core contraction gave up"
-                 : (err & 2) ? "non-finite values met in a truncation"
-                             : "a Jacobi eigen-solve hit its sweep limit";
+      j->status = flag_status(err);
+      j->error = get_error();
       ok = false;
     }
   }

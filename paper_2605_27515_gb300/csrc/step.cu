@@ -1123,23 +1123,34 @@ qlb_status run_steps(qlb_state* st, int64_t n, bool sync) {
   return check_flags(st);
 }
 
-// The state's device error flags and trace after its work has completed.
-qlb_status check_flags(qlb_state* st) {
+// A status and message for the error flags that the kernels of a step set; the first cause
+// wins, as a lost wait leaves values that trip the other checks.
+qlb_status flag_status(int err) {
+  if (err & 4) {
+    set_error("a bounded wait inside a truncation solve or a tensor-core contraction gave up");
+    return QLB_ETIMEOUT;
+  }
+  if (err & 2) {
+    set_error("non-finite values met in a truncation");
+    return QLB_ENONFINITE;
+  }
+  if (!err) return QLB_OK;
+  set_error("a Jacobi eigen-solve hit its sweep limit");
+  return QLB_ENOTCONV;
+}
+
+// Reads and clears the state's device error flags.
+static qlb_status take_flags(qlb_state* st) {
   int err = 0;
   QLB_CUDA_TRY(cudaMemcpy(&err, st->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {
-    QLB_CUDA_TRY(cudaMemset(st->d_err, 0, sizeof(int)));
-    if (err & 4) {
-      set_error("a bounded wait of the tensor-core contraction gave up");
-      return QLB_ETIMEOUT;
-    }
-    if (err & 2) {
-      set_error("non-finite values met in a truncation");
-      return QLB_ENONFINITE;
-    }
-    set_error("a Jacobi eigen-solve hit its sweep limit");
-    return QLB_ENOTCONV;
-  }
+  if (err) QLB_CUDA_TRY(cudaMemset(st->d_err, 0, sizeof(int)));
+  return flag_status(err);
+}
+
+// The state's device error flags and trace after its work has completed.
+qlb_status check_flags(qlb_state* st) {
+  qlb_status s = take_flags(st);
+  if (s) return s;
   double stats[2];
   QLB_CUDA_TRY(cudaMemcpy(stats, st->d_stats, sizeof(stats), cudaMemcpyDeviceToHost));
   if (!std::isfinite(stats[1])) {
@@ -1157,14 +1168,7 @@ qlb_status truncate_pass(qlb_state* st) {
   if ((s = enqueue_step(st, st->kraus_id, false))) return s;
   qlb_ctx* ctx = st->sys->ctx;
   QLB_CUDA_TRY(cudaStreamSynchronize(st->stream));
-  int err = 0;
-  QLB_CUDA_TRY(cudaMemcpy(&err, st->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {
-    QLB_CUDA_TRY(cudaMemset(st->d_err, 0, sizeof(int)));
-    set_error(err & 2 ? "non-finite values met in a truncation" : "a Jacobi eigen-solve hit its sweep limit");
-    return err & 2 ? QLB_ENONFINITE : QLB_ENOTCONV;
-  }
-  return QLB_OK;
+  return take_flags(st);
 }
 
 // ------------------------------------------------------------------ observables

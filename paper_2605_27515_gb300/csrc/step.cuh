@@ -24,6 +24,8 @@ qlb_status state_sum_abs2_site0(qlb_state* st, double* out);
 qlb_status run_steps(qlb_state* st, int64_t n, bool sync);
 // The state's device error flags and trace, read after its work has completed.
 qlb_status check_flags(qlb_state* st);
+// The status (and the thread's error text) of a set of device error flags.
+qlb_status flag_status(int err);
 
 // The captured step of a group of states (one launch per position over all members).
 struct GroupExec {

@@ -83,6 +83,7 @@ _SIGS = {
     "qlb_eig_check": (_st, [C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_double), C.c_double, C.c_int,
                             C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_int),
                             C.POINTER(C.c_double)]),
+    "qlb_inject_flags": (_st, [_vp, C.c_int]),
     "qlb_lost_wait_check": (_st, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int]),
     "qlb_system_create": (_st, [_vp, C.c_int, C.POINTER(C.c_int), C.POINTER(_vp)]),
     "qlb_system_destroy": (None, [_vp]),
@@ -421,6 +422,9 @@ class State:
         _check(self.lib.qlb_kraus_to_dense(self.h, float(dt), int(k), out.ctypes.data_as(C.POINTER(C.c_double)),
                                            2 * N * N))
         return out
+
+    def inject_flags(self, flags):
+        _check(self.lib.qlb_inject_flags(self.h, int(flags)))
 
     def export(self) -> bytes:
         n = C.c_size_t()
