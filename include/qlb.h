@@ -445,6 +445,18 @@ qlb_status qlb_zgemm_check(int device, int engine, int m, int n, int k, const do
 qlb_status qlb_eig_check(int device, int precision, int solver, int n, const double* G, double tol, int cap,
                          double* lam, double* V, int* k_out, double* ms);
 
+/* The truncated SVD of the operator builder (Sec. II.B) on a host matrix, exposed so that its
+ * numerics and its memory can be checked on their own.
+ *   A          m x n row-major complex128 (2 m n doubles)
+ *   tol, cap   relative discarded weight; cap on k (<= 0: none)
+ *   u_scale    0: U has orthonormal columns; 1: they carry the singular values
+ *   r_unscale  0: the rows of R carry the singular values; 1: R has orthonormal rows
+ *   U, R       m x k and k x n row-major (room for 2 m min(m, n) and 2 min(m, n) n doubles);
+ *              U R = A up to the cut when exactly one of them carries the singular values
+ * Device memory comes from the context, within its hbm_budget. */
+qlb_status qlb_svd_check(qlb_ctx* ctx, int m, int n, const double* A, double tol, int cap, int u_scale,
+                         int r_unscale, double* U, double* R, int* k_out);
+
 /* Failure injection on the host: sets the error flags that the kernels of a state's next
  * call may set, so that the call reports them: 1 a solve hit its sweep limit
  * (QLB_ENOTCONV), 2 non-finite values (QLB_ENONFINITE), 4 a bounded wait gave up

@@ -1136,6 +1136,34 @@ QLB_API qlb_status qlb_eig_check(int device, int precision, int solver, int n, c
   return eig_check(device, precision, solver, n, G, tol, cap, lam, V, k_out, ms, 0);
 }
 
+// ------------------------------------------------------------------ operator SVD check
+
+QLB_API qlb_status qlb_svd_check(qlb_ctx* ctx, int m, int n, const double* A, double tol, int cap, int u_scale,
+                                 int r_unscale, double* U, double* R, int* k_out) {
+  CHECK_ARG(ctx && A && U && R && k_out, "null argument");
+  CHECK_ARG(m >= 1 && n >= 1 && (long)m * n <= (1L << 24), "sizes out of range");
+  CHECK_ARG(tol >= 0 && tol < 1, "tol must be in [0, 1)");
+  zd *X = nullptr, *dU = nullptr, *dR = nullptr;
+  const size_t bytes = sizeof(zd) * (size_t)m * n;
+  qlb_status s = dev_alloc(ctx, (void**)&X, bytes);
+  if (s) return s;
+  int k = 0;
+  cudaError_t e = cudaMemcpyAsync(X, A, bytes, cudaMemcpyHostToDevice, ctx->stream);
+  if (e == cudaSuccess) s = svd_osj(ctx, X, m, n, tol, cap, &dU, u_scale, &dR, r_unscale, &k, 60);
+  if (e == cudaSuccess && !s) {
+    e = cudaMemcpyAsync(U, dU, sizeof(zd) * (size_t)m * k, cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(R, dR, sizeof(zd) * (size_t)k * n, cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  }
+  dev_free(ctx, X);
+  dev_free(ctx, dU);
+  dev_free(ctx, dR);
+  QLB_CUDA_TRY(e);
+  *k_out = k;
+  return s;
+}
+
 // ------------------------------------------------------------------ lost-wait check
 
 // The operator SVD of the n x 4n matrix M in one launch, with CTA `cta` stalled.

@@ -309,7 +309,10 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
     std::swap(m, n);
   }
   // the factors are at most min(m, n) = m wide
-  if ((st = dev_alloc_queued(ctx, &bt.p, sizeof(zd) * (size_t)m * m)) || (st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double))) ||
+  const bool one_launch = osj_serves(m, n);
+  const size_t coef = tall && !one_launch ? 2 * (size_t)(m + 1) : 0;
+  if ((st = dev_alloc_queued(ctx, &bt.p, sizeof(zd) * (size_t)m * m)) ||
+      (st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double) + sizeof(zd) * coef)) ||
       (st = dev_alloc_queued(ctx, &bu.p, sizeof(zd) * (size_t)(tall ? n : m) * m)) ||
       (st = dev_alloc_queued(ctx, &br.p, sizeof(zd) * (size_t)m * (tall ? m : n))))
     return st;
@@ -317,7 +320,7 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   int* d_cnt = (int*)bc.p;  // sweeps or rotations, then the kept count
   const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, tall, (zd*)bu.p, (zd*)br.p, d_cnt + 1, 0};
   int h[2] = {0, 0};
-  if (osj_serves(m, n)) {
+  if (one_launch) {
     QLB_CUDA_TRY(launch_osj(X, m, n, T, max_sweeps, d_cnt, out, s));
   } else {
     double* d_thr = (double*)d_cnt + 1;
@@ -338,7 +341,7 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
       return QLB_ENOTCONV;
     }
     cudaMemsetAsync(d_cnt, 1, sizeof(int), s);  // converged
-    QLB_CUDA_TRY(launch_osj_finish(X, m, n, T, out, s));
+    QLB_CUDA_TRY(launch_osj_finish(X, m, n, T, (zd*)((double*)d_cnt + 4), out, s));
   }
   cudaMemcpyAsync(h, d_cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);

@@ -78,8 +78,8 @@ struct OsjOut {
 bool osj_serves(int m, int n);
 // all sweeps on the rows of X (m x n; may be overwritten, like T, m x m) and the factors
 cudaError_t launch_osj(zd* X, int m, int n, zd* T, int max_sweeps, int* sweeps_out, const OsjOut& out, cudaStream_t s);
-// the factors alone, from rotated rows X and the rotations T
-cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, const OsjOut& out, cudaStream_t s);
+// the factors alone, from rotated rows X and the rotations T; coef: 2 (m + 1) entries of scratch if tall
+cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, zd* coef, const OsjOut& out, cudaStream_t s);
 void init_osj_attributes();
 qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** U, int u_scale, zd** Rr,
                    int r_unscale, int* k_out, int max_sweeps);

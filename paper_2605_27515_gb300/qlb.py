@@ -83,6 +83,8 @@ _SIGS = {
     "qlb_eig_check": (_st, [C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_double), C.c_double, C.c_int,
                             C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_int),
                             C.POINTER(C.c_double)]),
+    "qlb_svd_check": (_st, [_vp, C.c_int, C.c_int, C.POINTER(C.c_double), C.c_double, C.c_int, C.c_int, C.c_int,
+                            C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_int)]),
     "qlb_inject_flags": (_st, [_vp, C.c_int]),
     "qlb_lost_wait_check": (_st, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int]),
     "qlb_system_create": (_st, [_vp, C.c_int, C.POINTER(C.c_int), C.POINTER(_vp)]),
@@ -493,6 +495,18 @@ def qlb_eig_check(device: int, precision: int, solver: int, G, tol: float = 0.0,
                                 C.byref(ms)))
     kk = k.value
     return lam, (V[:n * kk].reshape(n, kk) if kk > 0 else None), kk, ms.value
+
+
+def qlb_svd_check(ctx: Ctx, A, tol: float = 0.0, cap: int = 0, u_scale: bool = False, r_unscale: bool = False):
+    """The operator builder's truncated SVD of A: (U, R) with A = U R up to the cut."""
+    A = np.ascontiguousarray(np.asarray(A, dtype=np.complex128))
+    m, n = A.shape
+    U, R = np.zeros(m * min(m, n), dtype=np.complex128), np.zeros(min(m, n) * n, dtype=np.complex128)
+    k = C.c_int()
+    dp = C.POINTER(C.c_double)
+    _check(ctx.lib.qlb_svd_check(ctx.h, m, n, A.ctypes.data_as(dp), float(tol), int(cap), int(u_scale),
+                                 int(r_unscale), U.ctypes.data_as(dp), R.ctypes.data_as(dp), C.byref(k)))
+    return U[:m * k.value].reshape(m, k.value), R[:k.value * n].reshape(k.value, n)
 
 
 WAIT_FACTOR, WAIT_EXCHANGE, WAIT_RANGE, WAIT_SVD = range(4)

@@ -1,0 +1,77 @@
+"""The operator builder's SVD on its own (qlb_svd_check): orthonormal factors and U R = A on tall
+and wide matrices whose rows or columns are graded down to, and past, the rounding level.
+
+Bars: U or R holds vectors of up to 520 entries, each rotated fewer than 6 * 520 times or
+projected twice, so 40 k eps bounds their loss of orthogonality as in the other solver tests;
+1e-12 relative Frobenius for U R (rotations' roundings, as for whole operators)."""
+import numpy as np
+import pytest
+
+from paper_2605_27515_gb300 import qlb as Q
+
+pytestmark = pytest.mark.gpu
+
+EPS = 2.220446049250313e-16
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = Q.Ctx(device=0)
+    yield c
+    c.close()
+
+
+def _unitary(rng, n, k):
+    return np.linalg.qr(rng.normal(size=(n, k)) + 1j * rng.normal(size=(n, k)))[0]
+
+
+def _graded(m, n, decades, seed):
+    """Singular values falling evenly over `decades`."""
+    rng = np.random.default_rng(seed)
+    k = min(m, n)
+    return (_unitary(rng, m, k) * np.logspace(0, -decades, k)) @ _unitary(rng, n, k).conj().T
+
+
+def _deficient(m, n, rank, seed):
+    """Exact rank `rank` up to rounding, as the stacked cores of a sum of operators have."""
+    rng = np.random.default_rng(seed)
+    return rng.normal(size=(m, rank)) @ (rng.normal(size=(rank, n)) + 1j * rng.normal(size=(rank, n)))
+
+
+SHAPES = [(4, 1), (8, 2), (40, 10), (64, 16), (41, 40), (172, 43), (1000, 12), (3000, 100), (560, 520)]
+CASES = ["graded 14", "graded 30", "rank 1", "rank half", "equal columns"]
+
+
+def _matrix(m, n, case, seed=3):
+    if case.startswith("graded"):
+        return _graded(m, n, int(case.split()[1]), seed)
+    if case == "equal columns":
+        return np.repeat(_graded(m, 1, 0, seed), n, axis=1)
+    return _deficient(m, n, 1 if case == "rank 1" else max(1, min(m, n) // 2), seed)
+
+
+def _check(ctx, A, u_scale, tol):
+    U, R = Q.qlb_svd_check(ctx, A, tol=tol, u_scale=u_scale, r_unscale=u_scale)
+    k = U.shape[1]
+    assert 1 <= k <= min(A.shape)
+    assert np.linalg.norm(U @ R - A) <= 1e-12 * np.linalg.norm(A)
+    return U, R, k
+
+
+@pytest.mark.parametrize("tol", [1e-32, 0.0])
+@pytest.mark.parametrize("case", CASES)
+@pytest.mark.parametrize("m,n", SHAPES)
+def test_tall_left_factor_is_orthonormal(ctx, m, n, case, tol):
+    """The left factor of a left-canonical sweep (singular values in R)."""
+    U, R, k = _check(ctx, _matrix(m, n, case), False, tol)
+    assert np.max(np.abs(U.conj().T @ U - np.eye(k))) <= 40 * k * EPS
+
+
+@pytest.mark.parametrize("case", CASES)
+@pytest.mark.parametrize("m,n", [(64, 16), (16, 64), (172, 43), (43, 172)])
+def test_unitary_side(ctx, m, n, case):
+    """The factor that the accumulated rotations give: U of a wide matrix, R of a tall one."""
+    tall = m > n
+    U, R, k = _check(ctx, _matrix(m, n, case), tall, 1e-32)
+    Z = R.conj().T if tall else U
+    assert np.max(np.abs(Z.conj().T @ Z - np.eye(k))) <= 40 * k * EPS
