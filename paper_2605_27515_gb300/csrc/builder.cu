@@ -302,21 +302,23 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
     ~Buf() { dev_free(c, p); }
   } xt{ctx}, bt{ctx}, bc{ctx}, bu{ctx}, br{ctx};
   qlb_status st;
+  zd* T = nullptr;  // the rotations, m x m of the rotated side
   if (tall) {
     if ((st = dev_alloc_queued(ctx, &xt.p, sizeof(zd) * (size_t)m * n))) return st;
     k_conj_transpose<<<nblk((long)m * n), 256, 0, s>>>(X, (zd*)xt.p, m, n);
+    T = X;  // done with: n x n of its m x n, so that a tall matrix takes no more memory than rotating its rows
     X = (zd*)xt.p;
     std::swap(m, n);
   }
   // the factors are at most min(m, n) = m wide
   const bool one_launch = osj_serves(m, n);
   const size_t coef = tall && !one_launch ? 2 * (size_t)(m + 1) : 0;
-  if ((st = dev_alloc_queued(ctx, &bt.p, sizeof(zd) * (size_t)m * m)) ||
+  if ((!tall && (st = dev_alloc_queued(ctx, &bt.p, sizeof(zd) * (size_t)m * m))) ||
       (st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double) + sizeof(zd) * coef)) ||
       (st = dev_alloc_queued(ctx, &bu.p, sizeof(zd) * (size_t)(tall ? n : m) * m)) ||
       (st = dev_alloc_queued(ctx, &br.p, sizeof(zd) * (size_t)m * (tall ? m : n))))
     return st;
-  zd* T = (zd*)bt.p;
+  if (!tall) T = (zd*)bt.p;
   int* d_cnt = (int*)bc.p;  // sweeps or rotations, then the kept count
   const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, tall, (zd*)bu.p, (zd*)br.p, d_cnt + 1, 0};
   int h[2] = {0, 0};

@@ -75,3 +75,14 @@ def test_unitary_side(ctx, m, n, case):
     U, R, k = _check(ctx, _matrix(m, n, case), tall, 1e-32)
     Z = R.conj().T if tall else U
     assert np.max(np.abs(Z.conj().T @ Z - np.eye(k))) <= 40 * k * EPS
+
+
+@pytest.mark.parametrize("m,n", [(40, 39), (39, 40), (64, 16), (300, 250)])
+def test_memory(m, n):
+    """Device memory beside the matrix: at most the rotations and a left factor of m x m and a
+    right factor of m x n (and 4 KB of counts and scratch), the budget the rows' own rotation needs."""
+    budget = 16 * (2 * m * n + 2 * m * m) + 4096
+    c = Q.Ctx(device=0, hbm_budget=budget)
+    U, R = Q.qlb_svd_check(c, _graded(m, n, 3, 1), tol=1e-32)
+    assert U.shape[1] == min(m, n)
+    c.close()
