@@ -38,7 +38,8 @@ constexpr size_t OSJ_SMEM_LIMIT = 200 * 1024;
 // cost its 64 clocks a warp each.  Truncated; zero below FP32's normal range, infinite above.
 __device__ __forceinline__ float osj_to_f(double v, int k) {
   const unsigned hi = (unsigned)__double2hiint(v);
-  const int e = (int)((hi >> 20) & 0x7ff) + k - 896;
+  const int ev = (int)((hi >> 20) & 0x7ff);
+  const int e = ev ? ev + k - 896 : 0;  // zero (and subnormal) stays zero whatever k
   const unsigned b = (hi & 0x80000000u) | ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | ((unsigned)__double2loint(v) >> 29);
   return __uint_as_float(e <= 0 ? 0u : e >= 255 ? (hi & 0x80000000u) | 0x7f800000u : b);
 }
@@ -49,8 +50,8 @@ __device__ __forceinline__ double osj_to_d(float f) {
 }
 // v 2^k for a normal result (zero below)
 __device__ __forceinline__ double osj_scale(double v, int k) {
-  const int hi = __double2hiint(v);
-  return ((hi >> 20) & 0x7ff) + k <= 0 ? 0.0 : __hiloint2double(hi + k * (1 << 20), __double2loint(v));
+  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+  return !e || e + k <= 0 ? 0.0 : __hiloint2double(hi + k * (1 << 20), __double2loint(v));
 }
 
 __device__ __forceinline__ int osj_player(int pos, int round, int np) {

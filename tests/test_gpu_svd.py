@@ -86,3 +86,20 @@ def test_memory(m, n):
     U, R = Q.qlb_svd_check(c, _graded(m, n, 3, 1), tol=1e-32)
     assert U.shape[1] == min(m, n)
     c.close()
+
+
+@pytest.mark.parametrize("power", [0, -440, -455, -500, 455])
+@pytest.mark.parametrize("m,n", [(2, 3), (9, 20), (20, 9), (40, 40)])
+def test_orthogonal_rows_of_any_size(ctx, m, n, power):
+    """Rows without a common entry, one of them zero: their couplings are exact zeros, so nothing is
+    rotated however small the entries are (squares down to 2^-1000), and the factors are exact."""
+    rng = np.random.default_rng(m + n)
+    A = np.zeros((m, n), dtype=np.complex128)
+    d = min(m, n)
+    A[np.arange(d), rng.permutation(n)[:d]] = np.arange(2.0, d + 2.0) * 2.0 ** power
+    A[d // 2] = 0.0
+    U, R = Q.qlb_svd_check(ctx, A)
+    assert U.shape[1] == d - 1
+    np.testing.assert_array_equal(U @ R, A)
+    np.testing.assert_array_equal(np.sort(np.abs(U), axis=0)[-1], 1.0)
+    assert np.count_nonzero(U) == d - 1
