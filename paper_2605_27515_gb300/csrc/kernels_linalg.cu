@@ -8,18 +8,19 @@
 // complex products takes one SM 16 us, a 16 x 16 x 16 block 4 us, an 8 x 8 x 16 block 1 us.
 // The kernel is persistent over a fixed grid (at most four CTAs per SM) and decides the
 // decomposition at run time from the actual sizes: output tiles of 16 x 16 or 8 x 8 (the
-// eight warps of a CTA take a quarter of the K chunk each), whichever finishes first with
-// its padding counted, and, with a workspace, a split of the K range into s parts while
-// tiles are fewer than CTAs and a part still outweighs what adding the parts costs.  Each
+// eight warps of a CTA take a quarter of the K chunk each), whichever finishes first, or takes
+// less work in all, with its padding counted, and, with a workspace, a split of the K range into s
+// parts while tiles are fewer than CTAs and a part still outweighs what adding the parts costs.  Each
 // (tile, part) item writes its partial tile to the workspace; the CTA that finishes a
 // tile last (a per-tile counter, no waiting) adds the s partials in part order and applies
 // alpha and beta, so the result does not depend on timing.
 //
 // Measured on GB300 (C = A B, m x n x k; before: 32 x 32 tiles on two CTAs per SM, parts of 16
 // upwards): FP64 16 x 16 x 16 9 us (16), 20 x 32 x 14 9 us (19), 30 x 30 x 30 10 us (28),
-// 64^3 12 us (30), 60 x 60 x 2600 104 us (166), 128 x 128 x 600 103 us (100, of which the FP64
-// pipe needs 62); double-float 9 us (13), 8 us (16), 9 us (22), 11 us (21), 62 us (91), 55 us (52).
-// What is left of the small ones is the launch and a chain of three trips to L2.
+// 64^3 12 us (30), 60 x 60 x 2600 94 us (164), 128 x 128 x 600 89 us (100, of which the FP64
+// pipe needs 62), 512^3 0.94 ms (1.05); double-float 9 us (12), 8 us (16), 9 us (22), 11 us (21),
+// 45 us (91), 42 us (52), 0.35 ms (0.43).  What is left of the small ones is the launch and a chain
+// of three trips to L2.
 
 #include <algorithm>
 #include <type_traits>
@@ -157,7 +158,9 @@ __device__ void gemm_items(const GemmDesc& g, const int* d, const GemmPlan& P, i
     const bool work = wrow < P.m;
     cx<Cm> acc = mk<Cm>(GAcc<Cm>().value(), GAcc<Cm>().value());
     for (int k0 = kbeg; k0 < kend; k0 += GB_K) {
-      zd v[2 * NL];  // all loads of a chunk in flight (three CTAs per SM cover their latency)
+      // All loads of a chunk in flight.  Up to three CTAs per SM cover their latency for each other;
+      // where a launch has one (most of a step's), nothing does.
+      zd v[2 * NL];
 #pragma unroll
       for (int q = 0; q < NL; q++) {
         const int e = tid + q * G_THREADS;
@@ -285,12 +288,25 @@ __global__ void __launch_bounds__(G_THREADS, 3) k_gemm(const GemmDesc g_in, cons
   P.nb2 = dev_eval(g.nb2, d);
   const int nb = P.nb1 * P.nb2;
   if (P.m <= 0 || P.n <= 0 || nb <= 0) return;
+  // Most CTAs of a small product find no work however it is cut (parts are of 32 in K at least) and
+  // leave before the plan: 16 cats of N = 32 at bonds of 1, on their own streams, are bound by it.
+  const long t8 = (long)((P.m + 7) / 8) * ((P.n + 7) / 8) * nb;
+  if (blockIdx.x && (long)blockIdx.x >= t8 * max(1, (P.K + 31) / 32)) return;
   // the tile: both counts of tiles in waves over the SMs (a quarter of the nominal grid)
   const long t16 = (long)((P.m + 15) / 16) * ((P.n + 15) / 16) * nb;
-  const long t8 = (long)((P.m + 7) / 8) * ((P.n + 7) / 8) * nb;
   const int sms = max(1, gnom / 4);
-  const float c16 = (float)((t16 + sms - 1) / sms) * tile_cycles<Cm>(16, P.K);
-  const float c8 = (float)((t8 + sms - 1) / sms) * tile_cycles<Cm>(8, P.K);
+  // Products that keep the chip busy however they are cut go by their work with its padding: a
+  // product takes an SM 2.0 cycles in tiles of 16 and 2.4 in tiles of 8, which read shared memory
+  // twice as often, in double-float 0.75 and 1.2 (768^3).  The others go by waves over the SMs.
+  // About the line, tiles of 16 against 8: 150^3 41 us against 44, double-float 30 against 25;
+  // 128 x 128 x 600 90 against 102, 40 against 57; 256^3 146 against 148, 64 against 74; 512^3 0.94 ms
+  // against 1.10, 0.35 against 0.53.  A Gram matrix's line lies higher: in a step, behind the
+  // launch that wrote its operand, 162 x 162 x 496 is 50 us slower in tiles of 16.
+  const float products = (float)P.m * (float)P.n * (float)P.K * (float)nb;
+  const bool large = products >= (g.kclass == QLB_K_GRAM ? 1.6e7f : 8.0e6f);
+  const float c16 = large ? (std::is_same<Cm, double>::value ? 4.f * 0.83f : 4.f * 0.63f) * (float)t16
+                          : (float)((t16 + sms - 1) / sms) * tile_cycles<Cm>(16, P.K);
+  const float c8 = large ? (float)t8 : (float)((t8 + sms - 1) / sms) * tile_cycles<Cm>(8, P.K);
   const bool small = c8 < c16;
   P.ntiles = small ? t8 : t16;
   P.tm = small ? (P.m + 7) / 8 : (P.m + 15) / 16;
@@ -302,6 +318,13 @@ __global__ void __launch_bounds__(G_THREADS, 3) k_gemm(const GemmDesc g_in, cons
   if (g.ws && P.K > least && P.ntiles < (long)gnom) {
     const int cap = g.ksplit >= 1 ? g.ksplit : GB_SPLIT_CAP;
     P.ks = (int)min((long)cap, (long)gnom / P.ntiles);
+    if (large) {
+      // Three of the nominal four CTAs per SM are resident: parts that fill their places leave no
+      // second wave (192 x 192 x 2048: 568 us in 3 parts, 680 in 4), but a grid part empty is spread
+      // unevenly (162 x 162 x 496, 121 tiles: 165 us in 3 parts, 113 in 4).
+      const int slots = 3 * sms, per = slots / (int)P.ntiles;
+      if (16 * per * (int)P.ntiles >= 15 * slots) P.ks = min(P.ks, per);
+    }
     P.ks = max(1, min(P.ks, (P.K + least - 1) / least));
   }
   P.chunk = P.ks > 1 ? (((P.K + P.ks - 1) / P.ks + GB_K - 1) / GB_K) * GB_K : P.K;
