@@ -392,9 +392,10 @@ qlb_status qlb_profile_reset(qlb_ctx* ctx);
  * Synchronises the device. */
 qlb_status qlb_profile_solver_stats(qlb_ctx* ctx, double* out, int n_out);
 
-/* Autotuner of the step's launch shapes: times the zip-up Gram GEMM at split-K
- * factors 1, 2, 4, 8, 16 for every (rows, inner size) bucket with CUDA events on
- * random data, installs the fastest in the context (used by every state planned
+/* Autotuner of the step's launch shapes: times the zip-up Gram GEMM, launched as a step
+ * does, with its split-K capped at 64 (the kernel's own cap), 32, 16, 8, 4, 2 and 1 for
+ * every (rows, inner size) bucket with CUDA events on random data, installs the largest cap
+ * that no smaller one beats by 3 % in the context (used by every state planned
  * afterwards) and, when path is non-NULL, writes the table as lines "m K ksplit".
  * Allocates scratch for the duration of the call.  The paper has no counterpart. */
 qlb_status qlb_autotune(qlb_ctx* ctx, const char* path);

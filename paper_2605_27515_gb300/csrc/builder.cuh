@@ -19,6 +19,7 @@ cudaError_t launch_gemm(const GemmDesc& g, const int* d_dims, cudaStream_t s, do
 // its counters must start at zero), and the default grid (four CTAs per SM)
 size_t gemm_workspace_elems(int grid);
 int gemm_grid_default();
+int step_gemm_ctas(int kclass, int m_max);
 template <typename R>
 cudaError_t launch_eig(const EigDesc& e, const int* d_dims, cudaStream_t s, void* work, double* prof);
 template <typename R>

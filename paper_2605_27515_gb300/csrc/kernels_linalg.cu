@@ -362,6 +362,17 @@ int gemm_grid_default() {
   return grid;
 }
 
+// CTAs that a step launches for a GEMM of m_max planned rows (GemmDesc::ctas): one per SM, four
+// for a Gram matrix planned above 64.  The sizes that a launch meets are mostly far below the
+// planned ones, and states on their own streams share the SMs: sixteen cats of N = 32 at bonds of 1
+// took 0.97 ms a step of all with four for every GEMM, 0.55 with this rule, and 0.49 now that CTAs
+// without work leave before the plan.  One for the large Grams costs 6 % of their time in the
+// transmon at chi 128 (6.21 ms in two steps against 5.85) and 12 % in the coupled cats (4.31
+// against 3.84), two cost 4 and 7 %.  The tiles and the K split stay those of the full grid.
+int step_gemm_ctas(int kclass, int m_max) {
+  return kclass == QLB_K_GRAM && m_max > 64 ? 0 : gemm_grid_default() / 4;
+}
+
 cudaError_t launch_gemm(const GemmDesc& g, const int* d_dims, cudaStream_t s, double* prof) {
   const long planned =
       (long)((g.m_max + 7) / 8) * ((g.n_max + 7) / 8) * (g.nb_max > 0 ? g.nb_max : 1);

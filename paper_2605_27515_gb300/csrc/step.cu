@@ -242,12 +242,7 @@ static inline void debug_dump(qlb_state*, int, const void*) {}
 static qlb_status gemm(qlb_state* st, GemmDesc& g) {
   qlb_ctx* ctx = st->sys->ctx;
   if (!g.ws && st->Wsk && st->nWsk >= gemm_workspace_elems(gemm_grid_default())) g.ws = st->Wsk;
-  // One CTA per SM, four for a Gram matrix planned above 64: the sizes that a launch meets are mostly
-  // far below the planned ones, and states on their own streams share the SMs.  Sixteen cats of
-  // N = 32 at bonds of 1 step in 0.97 ms with four each (the placing of CTAs that find no work) and
-  // 0.53 with this rule; the largest steps lose under 1 %.  The tiles and the K split stay those of the
-  // full grid.
-  g.ctas = g.kclass == QLB_K_GRAM && g.m_max > 64 ? 0 : gemm_grid_default() / 4;
+  g.ctas = step_gemm_ctas(g.kclass, g.m_max);
   // the mixed forms multiply in double-float (FP64 operands and results)
   if (st->prec != QLB_PREC_F64)
     g.df64 = ctx->opt.mixed_gemm >= 2 || (ctx->opt.mixed_gemm == 1 && g.kclass != QLB_K_GRAM);

@@ -2,10 +2,12 @@
 // the zip-up Gram GEMM G = M M^dag, whose (2z) x (2z) output makes few tiles
 // over a long K = d D (the work-distributed GEMM splits K until its fixed grid is
 // full; more parts mean more partial tiles to add).  For every bucket (rows m,
-// inner size K) the tuner times the GEMM with caps 1, 2, 4, 8, 16 with CUDA events
-// (best of three, on random data in a scratch allocation) and keeps the fastest;
-// the table lives in the context and can be written to / read from a text file of
-// lines "m K ksplit", so a tuning run on one GPU serves later runs.
+// inner size K) the tuner times the GEMM, on as many CTAs as a step launches, with caps 64
+// (the kernel's own), 32, 16, 8, 4, 2 and 1 with CUDA events (best of seven, on random data in a
+// scratch allocation) and keeps the largest that no smaller one beats by 3 %: a cap binds
+// at the smaller sizes of its bucket too, where more parts are wanted.  The table lives in
+// the context and can be written to / read from a text file of lines "m K ksplit", so a
+// tuning run on one GPU serves later runs.
 
 #include <algorithm>
 #include <cstdio>
@@ -22,7 +24,7 @@ namespace {
 
 const int kTuneM[] = {32, 64, 128, 256};
 const int kTuneK[] = {256, 1024, 4096};
-const int kTuneSplit[] = {1, 2, 4, 8, 16};
+const int kTuneSplit[] = {64, 32, 16, 8, 4, 2, 1};
 
 int bucket_m(long m) {
   for (int b : kTuneM)
@@ -84,7 +86,7 @@ QLB_API qlb_status qlb_autotune(qlb_ctx* ctx, const char* path) {
   for (int m : kTuneM)
     for (int K : kTuneK) {
       float best = 1e30f;
-      int best_ks = 1;
+      int best_ks = kTuneSplit[0];
       for (int ks : kTuneSplit) {
         GemmDesc g{};
         g.A = M;
@@ -100,10 +102,12 @@ QLB_API qlb_status qlb_autotune(qlb_ctx* ctx, const char* path) {
         g.alpha_re = 1.0;
         g.m_max = g.n_max = m;
         g.nb_max = 1;
+        g.kclass = QLB_K_GRAM;
+        g.ctas = step_gemm_ctas(g.kclass, m);
         g.ksplit = ks;
         g.ws = W;
         float t = 1e30f;
-        for (int rep = 0; rep < 4; rep++) {
+        for (int rep = 0; rep < 8; rep++) {
           cudaEventRecord(a, 0);
           cudaError_t e = launch_gemm(g, nullptr, 0, nullptr);
           cudaEventRecord(b, 0);
@@ -118,7 +122,7 @@ QLB_API qlb_status qlb_autotune(qlb_ctx* ctx, const char* path) {
           if (rep > 0) t = std::min(t, ms);  // the first launch warms up
         }
         if (st) break;
-        if (t < best) {
+        if (t < (best < 1e30f ? 0.97f : 1.f) * best) {
           best = t;
           best_ks = ks;
         }
@@ -137,7 +141,7 @@ QLB_API qlb_status qlb_autotune(qlb_ctx* ctx, const char* path) {
       set_error(std::string("qlb_autotune: cannot write ") + path);
       return QLB_EINVAL;
     }
-    fprintf(f, "# m K ksplit  (split-K of the Gram GEMM, fastest of 1 2 4 8 16 by CUDA events)\n");
+    fprintf(f, "# m K ksplit  (cap on the split-K of the Gram GEMM, of 64 32 16 8 4 2 1 by CUDA events)\n");
     for (auto& kv : table) fprintf(f, "%d %d %d\n", kv.first.first, kv.first.second, kv.second);
     fclose(f);
   }
