@@ -469,7 +469,7 @@ qlb_status qlb_inject_flags(qlb_state* st, int flags);
  * expecting an arrival that never comes, so that a bounded wait of a second runs out.
  *   kernel     0 the step's truncation solve, in its factorisation; 1 the same, in its
  *              exchanges of columns; 2 the zip-up range basis; 3 the operator builder's
- *              SVD (FP64 whatever the precision)
+ *              SVD, 4 the QR before it (on 4n x n; both FP64 whatever the precision)
  *   precision  QLB_PREC_F64 or QLB_PREC_MIXED
  * QLB_ETIMEOUT when the wait ran out and every CTA left, QLB_OK when fewer than cta + 1
  * CTAs work on this size (nothing waits for the missing arrival).  The device stays

@@ -1166,8 +1166,8 @@ QLB_API qlb_status qlb_svd_check(qlb_ctx* ctx, int m, int n, const double* A, do
 
 // ------------------------------------------------------------------ lost-wait check
 
-// The operator SVD of the n x 4n matrix M in one launch, with CTA `cta` stalled.
-static qlb_status osj_lost_wait(int device, int n, const std::vector<double>& M, int cta) {
+// The operator SVD of the n x 4n matrix M in one launch, or the QR of M as 4n x n, with CTA `cta` stalled.
+static qlb_status svd_lost_wait(int device, int n, const std::vector<double>& M, int cta, bool qr) {
   QLB_CUDA_TRY(cudaSetDevice(device));
   init_kernel_attributes();
   const size_t nn = (size_t)n * n;
@@ -1181,7 +1181,10 @@ static qlb_status osj_lost_wait(int device, int n, const std::vector<double>& M,
   const OsjOut out{1e-12, 1e-10, 0, 0, 0, 0, buf + 5 * nn, buf + 6 * nn, d_out + 1, cta + 1};
   int h = 0;
   cudaError_t e = cudaMemcpy(buf, M.data(), sizeof(zd) * 4 * nn, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = launch_osj(buf, n, 4 * n, buf + 4 * nn, 60, d_out, out, 0);
+  if (e == cudaSuccess)
+    e = qr ? launch_tall_qr(buf, 4 * n, n, 0, buf + 4 * nn, buf + 5 * nn, (double*)(buf + 6 * nn), d_out, d_out + 1,
+                            cta + 1, 0)
+           : launch_osj(buf, n, 4 * n, buf + 4 * nn, 60, d_out, out, 0);
   if (e == cudaSuccess) e = cudaMemcpy(&h, d_out, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(buf);
   QLB_CUDA_TRY(e);
@@ -1189,11 +1192,11 @@ static qlb_status osj_lost_wait(int device, int n, const std::vector<double>& M,
     set_error("qlb_lost_wait_check: a bounded wait between the SVD's CTAs gave up");
     return QLB_ETIMEOUT;
   }
-  return h > 0 ? QLB_OK : QLB_ENOTCONV;
+  return h > 0 || qr ? QLB_OK : QLB_ENOTCONV;
 }
 
 QLB_API qlb_status qlb_lost_wait_check(int device, int kernel, int precision, int n, int cta) {
-  CHECK_ARG(kernel >= 0 && kernel <= 3, "unknown kernel");
+  CHECK_ARG(kernel >= 0 && kernel <= 4, "unknown kernel");
   CHECK_ARG(n >= 1 && n <= 256, "n must be in [1, 256]");
   CHECK_ARG(cta >= 0 && cta < 16, "cta must be in [0, 16)");
   int ndev = 0;
@@ -1206,7 +1209,7 @@ QLB_API qlb_status qlb_lost_wait_check(int device, int kernel, int precision, in
   std::mt19937_64 rng(n);
   std::normal_distribution<double> nd;
   for (double& x : M) x = nd(rng);
-  if (kernel == 3) return osj_lost_wait(device, n, M, cta);
+  if (kernel >= 3) return svd_lost_wait(device, n, M, cta, kernel == 4);
   std::vector<double> G(2 * (size_t)n * n), V(G.size()), lam(n);  // M M^dag of the first n columns
   for (int i = 0; i < n; i++)
     for (int j = 0; j < n; j++) {

@@ -255,14 +255,6 @@ __global__ void k_zero(zd* p, long n) {
   if (x < n) p[x] = mk<double>(0, 0);
 }
 
-// B (n x m) = A^dag, A m x n
-__global__ void k_conj_transpose(const zd* A, zd* B, int m, int n) {
-  long x = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (x >= (long)m * n) return;
-  int i = (int)(x / n), j = (int)(x % n);
-  B[(long)j * m + i] = cconj(A[x]);
-}
-
 __global__ void k_abs_rowsum_max(const zd* A, int N, double* out) {
   __shared__ double sh[32];
   double best = 0;
@@ -291,38 +283,48 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
                    int r_unscale, int* k_out, int max_sweeps) {
   cudaStream_t s = ctx->stream;
   *U = *Rr = nullptr;
-  // The rows that are rotated are those of the matrix or of its conjugate transpose,
-  // whichever are fewer: a sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so
-  // the tall cores of a left-canonical sweep (4 D x D) cost a sixteenth (admission of an
-  // N = 64 cat, 135 such solves: 248 ms before, 48 with it).
-  const int tall = m > n;
+  // A tall matrix A = Q R goes through its triangular factor: R = T^dag X by rotating its n rows,
+  // so A = (Q T^dag) X with a left factor that is unitary to rounding whatever the singular values,
+  // or R^dag = T^dag X and A = (Q X^dag) T where the right factor is to be (Drmac & Veselic, "New fast and accurate Jacobi SVD algorithm I",
+  // 2008).  A sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so the tall cores of a
+  // left-canonical sweep (4 D x D) cost a fortieth of rotating their own rows (admission of an
+  // N = 64 cat, 135 SVDs: 248 ms with that on one CTA, 23 now), with the same operator ranks: the
+  // rows of A^dag instead of R's left rounding in U, which the recompression took for content
+  // (transmon and resonator: bonds of 13 or 15 where 12 and 11 are).
+  const int tall = m > n && n <= TALL_MAX_N;
   struct Buf {  // freed on return unless handed over
     qlb_ctx* c;
     void* p = nullptr;
     ~Buf() { dev_free(c, p); }
-  } xt{ctx}, bt{ctx}, bc{ctx}, bu{ctx}, br{ctx};
+    void release() {
+      dev_free(c, p);
+      p = nullptr;
+    }
+  } bx{ctx}, bt{ctx}, bc{ctx}, bu{ctx}, br{ctx};
   qlb_status st;
-  zd* T = nullptr;  // the rotations, m x m of the rotated side
-  if (tall) {
-    if ((st = dev_alloc_queued(ctx, &xt.p, sizeof(zd) * (size_t)m * n))) return st;
-    k_conj_transpose<<<nblk((long)m * n), 256, 0, s>>>(X, (zd*)xt.p, m, n);
-    T = X;  // done with: n x n of its m x n, so that a tall matrix takes no more memory than rotating its rows
-    X = (zd*)xt.p;
-    std::swap(m, n);
-  }
-  // the factors are at most min(m, n) = m wide
-  const bool one_launch = osj_serves(m, n);
-  const size_t coef = tall && !one_launch ? 2 * (size_t)(m + 1) : 0;
-  if ((!tall && (st = dev_alloc_queued(ctx, &bt.p, sizeof(zd) * (size_t)m * m))) ||
-      (st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double) + sizeof(zd) * coef)) ||
-      (st = dev_alloc_queued(ctx, &bu.p, sizeof(zd) * (size_t)(tall ? n : m) * m)) ||
-      (st = dev_alloc_queued(ctx, &br.p, sizeof(zd) * (size_t)m * (tall ? m : n))))
+  const int rows = tall ? n : m;  // rotated; the factors are at most that wide
+  const size_t r2 = sizeof(zd) * (size_t)rows * rows;
+  // counts, then the heads and factors of the reflectors
+  if ((st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double) + (tall ? (sizeof(zd) + sizeof(double)) * (size_t)n : 0))) ||
+      (st = dev_alloc_queued(ctx, &bt.p, r2)) || (tall && (st = dev_alloc_queued(ctx, &bx.p, r2))) ||
+      (!tall && (st = dev_alloc_queued(ctx, &bu.p, r2))) ||
+      (st = dev_alloc_queued(ctx, &br.p, sizeof(zd) * (size_t)rows * n)))
     return st;
-  if (!tall) T = (zd*)bt.p;
-  int* d_cnt = (int*)bc.p;  // sweeps or rotations, then the kept count
-  const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, tall, (zd*)bu.p, (zd*)br.p, d_cnt + 1, 0};
-  int h[2] = {0, 0};
-  if (one_launch) {
+  // sweeps or rotations, kept count, (a threshold,) [4] status of the QR
+  int* d_cnt = (int*)bc.p;
+  zd* const v0 = (zd*)((double*)bc.p + 4);
+  double* const tau = (double*)(v0 + n);
+  zd *const A = X, *const T = (zd*)bt.p;
+  const int am = m, dagger = tall && u_scale && r_unscale;
+  if (tall) {
+    X = (zd*)bx.p;
+    QLB_CUDA_TRY(launch_tall_qr(A, m, n, dagger, X, v0, tau, d_cnt + 4, d_cnt + 1, 0, s));
+    m = n;
+  }
+  zd* const small_u = dagger ? T : X;  // U of R, over what the right factor has been read from
+  const OsjOut out{tol, 1e-10, cap, u_scale, r_unscale, dagger, tall ? small_u : (zd*)bu.p, (zd*)br.p, d_cnt + 1, 0};
+  int h[5] = {0, 0, 0, 0, 0};
+  if (osj_serves(m, n)) {
     QLB_CUDA_TRY(launch_osj(X, m, n, T, max_sweeps, d_cnt, out, s));
   } else {
     double* d_thr = (double*)d_cnt + 1;
@@ -343,7 +345,12 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
       return QLB_ENOTCONV;
     }
     cudaMemsetAsync(d_cnt, 1, sizeof(int), s);  // converged
-    QLB_CUDA_TRY(launch_osj_finish(X, m, n, T, (zd*)((double*)d_cnt + 4), out, s));
+    QLB_CUDA_TRY(launch_osj_finish(X, m, n, T, out, s));
+  }
+  if (tall) {
+    (dagger ? bx : bt).release();  // (in the stream's order) so that U takes no more than rotating A's own rows did
+    if ((st = dev_alloc_queued(ctx, &bu.p, sizeof(zd) * (size_t)am * n))) return st;
+    QLB_CUDA_TRY(launch_tall_apply(A, am, n, v0, tau, small_u, d_cnt + 1, (zd*)bu.p, s));
   }
   cudaMemcpyAsync(h, d_cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);
@@ -351,7 +358,7 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
     set_error(std::string("svd finish: ") + cudaGetErrorString(e));
     return QLB_EDEVICE;
   }
-  if (h[0] == -2) {
+  if (h[0] == -2 || (tall && h[4] == -2)) {
     set_error("a bounded wait of the one-sided Jacobi SVD gave up");
     return QLB_ETIMEOUT;
   }

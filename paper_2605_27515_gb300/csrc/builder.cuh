@@ -67,11 +67,12 @@ template <typename R>
 cudaError_t launch_zipqr_group(int n_max, const EigDesc* d_grp, int S, cudaStream_t s, double* prof);
 void init_tc_attributes();
 
-// one-sided Jacobi SVD of the builder (kernels_osj.cu).  tall: X holds the rows of the
-// conjugate transpose of the matrix that was asked for, so U is n x k and Rr k x m
+// one-sided Jacobi SVD of the builder (kernels_osj.cu).  dagger: X holds the rows of the square
+// matrix's conjugate transpose, U carries the singular values and R has orthonormal rows.  U may lie
+// over what R is read from: X, or T if dagger.
 struct OsjOut {
   double tol, gap;
-  int cap, u_scale, r_unscale, tall;
+  int cap, u_scale, r_unscale, dagger;
   zd *U, *Rr;
   int* k_out;
   int stall;  // failure test: 1 + the CTA whose barrier expects an arrival that never comes
@@ -79,8 +80,19 @@ struct OsjOut {
 bool osj_serves(int m, int n);
 // all sweeps on the rows of X (m x n; may be overwritten, like T, m x m) and the factors
 cudaError_t launch_osj(zd* X, int m, int n, zd* T, int max_sweeps, int* sweeps_out, const OsjOut& out, cudaStream_t s);
-// the factors alone, from rotated rows X and the rotations T; coef: 2 (m + 1) entries of scratch if tall
-cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, zd* coef, const OsjOut& out, cudaStream_t s);
+// the factors alone, from rotated rows X and the rotations T
+cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, const OsjOut& out, cudaStream_t s);
+// columns of a tall matrix that goes through its QR (kernels_tallqr.cu: its rows' buffers)
+constexpr int TALL_MAX_N = 2048;
+// Householder QR of a tall matrix (kernels_tallqr.cu): A (m x n, m > n) becomes the reflectors
+// (below the diagonal; their heads v0 and factors tau aside) and R, or R^dag if dagger (n x n).
+// *status: 0, or -2 when a bounded wait gave up; *count: 0.  stall as in OsjOut.
+cudaError_t launch_tall_qr(zd* A, int m, int n, int dagger, zd* R, zd* v0, double* tau, int* status, int* count,
+                           int stall, cudaStream_t s);
+// U (m x k) = Q C for C of n x k, k read from device memory
+cudaError_t launch_tall_apply(const zd* A, int m, int n, const zd* v0, const double* tau, const zd* C, const int* k,
+                              zd* U, cudaStream_t s);
+void init_tallqr_attributes();
 void init_osj_attributes();
 qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** U, int u_scale, zd** Rr,
                    int r_unscale, int* k_out, int max_sweeps);

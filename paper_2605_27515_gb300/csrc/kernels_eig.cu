@@ -1115,6 +1115,7 @@ template cudaError_t launch_eig_kind<df64>(int, const EigDesc&, const int*, cuda
 void init_kernel_attributes() {
   init_pj_attributes();
   init_osj_attributes();
+  init_tallqr_attributes();
   cudaFuncSetAttribute(k_eig<double, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIG_SMEM_LIMIT);
   cudaFuncSetAttribute(k_eig<double, 512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIG_SMEM_LIMIT);
   cudaFuncSetAttribute(k_eig<df64, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIG_SMEM_LIMIT);

@@ -19,7 +19,8 @@
 // FP64 square roots and divisions, and the factors in a launch of their own): 16 x 16, ten sweeps,
 // 0.42 ms (1.30); 16 x 56 0.30 ms (0.86); 36 x 72, 13 sweeps, 2.0 ms (11.9, 14 sweeps);
 // 8 x 1,024 0.11 ms (0.52); 20 x 16,384 9.0 ms (110).  Admitting an N = 64 cat, 135 such
-// solves of 2 to 43 rows, 12 ms on the device: 47 ms before, 22 now.
+// solves of 2 to 43 rows, 12 ms on the device: 47 ms before, 22 with this kernel, 23 since tall
+// matrices go through their QR (kernels_tallqr.cu).
 
 #include <algorithm>
 
@@ -99,31 +100,17 @@ __device__ int osj_rule(double* w, double* ws, int* perm, int* s_k, int m, doubl
   return *s_k;
 }
 
-// our slice's part of the factors
-__device__ void osj_write(const OsjSlice& c, const double* sv, const double* inv, const int* perm, int m, int n, int k,
-                          const OsjOut& o) {
-  if (o.tall) {
-    // A^dag = T^dag X, so A = X^dag T: U[i, j] = conj(X[perm_j, i]) / s_j, R[j, :] = s_j T[perm_j, :]
-    // (the rows of X orthogonal as osj_orthonormalise leaves them)
-    for (long x = threadIdx.x; x < (long)c.nl * k; x += blockDim.x) {
-      const int i = (int)(x / k), j = (int)(x - (long)i * k);
-      zd v = cconj(c.x[perm[j] * c.ldx + i]);
-      if (!o.u_scale) v = sv[j] > 0 ? cscale(v, inv[j]) : mk<double>(c.j0 + i == j ? 1.0 : 0.0, 0);
-      o.U[(long)(c.j0 + i) * k + j] = v;
-    }
+// our slice's part of the factors: R[j, :] = X[perm_j, :] / s_j^r_unscale,
+// U[i, j] = conj(T[perm_j, i]) * s_j^u_scale; with X the rows of A^dag = T^dag X (A = X^dag T)
+// R[j, :] = T[perm_j, :], U[i, j] = conj(X[perm_j, i])
+__device__ void osj_write_r(const OsjSlice& c, const double* sv, const double* inv, const int* perm, int m, int n, int k,
+                            const OsjOut& o) {
+  if (o.dagger) {
     for (long x = threadIdx.x; x < (long)k * c.ml; x += blockDim.x) {
       const int j = (int)(x / c.ml), i = (int)(x - (long)j * c.ml);
-      const zd v = c.t[perm[j] * c.ldt + i];
-      o.Rr[(long)j * m + c.t0 + i] = o.r_unscale ? v : cscale(v, sv[j]);
+      o.Rr[(long)j * m + c.t0 + i] = c.t[perm[j] * c.ldt + i];
     }
     return;
-  }
-  // U[i, j] = conj(T[perm_j, i]) * s_j^u_scale,  R[j, :] = X[perm_j, :] / s_j^r_unscale
-  for (long x = threadIdx.x; x < (long)c.ml * k; x += blockDim.x) {
-    const int i = (int)(x / k), j = (int)(x - (long)i * k);
-    zd v = cconj(c.t[perm[j] * c.ldt + i]);
-    if (o.u_scale) v = cscale(v, sv[j]);
-    o.U[(long)(c.t0 + i) * k + j] = v;
   }
   for (long x = threadIdx.x; x < (long)k * c.nl; x += blockDim.x) {
     const int j = (int)(x / c.nl), i = (int)(x - (long)j * c.nl);
@@ -132,104 +119,20 @@ __device__ void osj_write(const OsjSlice& c, const double* sv, const double* inv
     o.Rr[(long)j * n + c.j0 + i] = v;
   }
 }
-
-// The rows of X that become orthonormal columns of U, made so where the sweeps leave them
-// short of it.  Rows are not rotated below the absolute floor, so rows p and q may overlap by
-// 1e-31 ||X||_F^2 / (s_p s_q) of their lengths: under 1e-15 while both stand above
-// 1e-8 ||X||_F, up to parallel ones at the rounding level.  Every kept row below that loses its
-// components along the ones before it (classical Gram-Schmidt, again while a pass takes more than
-// three quarters of the squared norm: "twice is enough", Giraud, Langou & Rozloznik 2005), and T
-// takes them up, so that U R stays the matrix: with u_i = x_i / s_i,
-//   x_q^dag t_q = sum_i conj(a_i) u_i^dag t_q + x'_q^dag t_q,   a_i = x_q u_i^dag.
-// A row of which three passes leave nothing is dropped, as the others hold all of it.
-//
-// w, ws, perm as osj_rule leaves them; returns the kept count.  coef: two sets of k + 1 entries
-// in turn (a set is written again behind the barrier that follows its reads).  Nothing to do
-// costs a sum over w; a row ~9,000 cycles, one barrier over the CTAs and three of the block.
-__device__ int osj_orthonormalise(const OsjSlice& c, double* w, double* ws, int* perm, int k, double f2, zd* coef0,
-                                  zd* coef1, ClusterBarrier& cb, bool update_t) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const long long thr = __double_as_longlong(1e-8 * ::sqrt(f2));  // lengths order like their bit patterns
-  int kk = 0;
-  for (int q0 = 0; q0 < k; q0 += 32)
-    kk += __popc(__ballot_sync(0xffffffffu, q0 + lane < k && __double_as_longlong(w[min(k - 1, q0 + lane)]) >= thr));
-  for (int q = kk; q < k; q++) {
-    const int row = perm[q];
-    zd* const xq = c.x + row * c.ldx;
-    const zd* const tq = c.t + row * c.ldt;
-    double left = 0.0;
-    bool done = false;
-    for (int pass = 0; pass < 3 && !done; pass++) {
-      // x_q . conj(x_i), and |x_q|^2 behind them
-      int G = 32;
-      while (G > 4 && ((kk + 1) * G > OSJ_NT || G >= 2 * c.nl)) G >>= 1;
-      const int g = tid / G, gl = tid % G, ng = OSJ_NT / G;
-      for (int i0 = 0; i0 <= kk; i0 += ng) {
-        const int i = i0 + g;
-        double re = 0.0, im = 0.0;
-        if (i <= kk) {
-          const zd* xi = i < kk ? c.x + perm[i] * c.ldx : xq;
-          for (int j = gl; j < c.nl; j += G) {
-            const zd u = xq[j], v = xi[j];
-            re = fma(u.im, v.im, fma(u.re, v.re, re));
-            im = fma(-u.re, v.im, fma(u.im, v.re, im));
-          }
-        }
-        for (int o = 1; o < G; o <<= 1) {
-          re += __shfl_xor_sync(0xffffffffu, re, o);
-          im += __shfl_xor_sync(0xffffffffu, im, o);
-        }
-        if (i <= kk && gl == 0) coef0[i] = mk<double>(re, im);
-      }
-      if (!cb.sync()) return k;
-      for (int i = tid; i <= kk; i += OSJ_NT) {
-        zd s = coef0[i];
-        if (cb.ca > 1) {
-          s = *on_cta(&coef0[i], 0);
-          for (int r = 1; r < cb.ca; r++) s = cadd(s, *on_cta(&coef0[i], r));
-        }
-        coef1[i] = i < kk ? cscale(s, ws[i]) : s;  // a_i
-      }
-      __syncthreads();
-      double gone = 0.0;
-      for (int i = lane; i < kk; i += 32) gone += cabs2(coef1[i]);
-      for (int o = 16; o > 0; o >>= 1) gone += __shfl_xor_sync(0xffffffffu, gone, o);
-      const double was = coef1[kk].re;
-      // x_q -= sum_i a_i u_i
-      for (int j0 = 0; j0 < c.nl; j0 += OSJ_NT / 8) {
-        const int j = j0 + tid / 8;
-        zd s = mk<double>(0.0, 0.0);
-        if (j < c.nl)
-          for (int i = tid & 7; i < kk; i += 8) cfma(s, cscale(coef1[i], ws[i]), c.x[perm[i] * c.ldx + j]);
-        for (int o = 1; o < 8; o <<= 1) {
-          s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
-          s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
-        }
-        if (j < c.nl && (tid & 7) == 0) xq[j] = csub(xq[j], s);
-      }
-      if (update_t)
-        for (int x = tid; x < kk * c.ml; x += OSJ_NT) {
-          const int i = x / c.ml, l = x - i * c.ml;
-          cfma(c.t[perm[i] * c.ldt + l], cscale(cconj(coef1[i]), ws[i]), tq[l]);
-        }
-      __syncthreads();
-      left = was - gone;
-      done = left > 0.0 && left >= 0.25 * was;
-      zd* const t = coef0;
-      coef0 = coef1;
-      coef1 = t;
+__device__ void osj_write_u(const OsjSlice& c, const double* sv, const int* perm, int k, const OsjOut& o) {
+  if (o.dagger) {
+    for (long x = threadIdx.x; x < (long)c.nl * k; x += blockDim.x) {
+      const int i = (int)(x / k), j = (int)(x - (long)i * k);
+      o.U[(long)(c.j0 + i) * k + j] = cconj(c.x[perm[j] * c.ldx + i]);
     }
-    if (done) {
-      if (tid == 0) {
-        perm[kk] = row;
-        w[kk] = ::sqrt(left);
-        ws[kk] = 1.0 / w[kk];
-      }
-      kk++;
-    }
-    __syncthreads();
+    return;
   }
-  return kk;
+  for (long x = threadIdx.x; x < (long)c.ml * k; x += blockDim.x) {
+    const int i = (int)(x / k), j = (int)(x - (long)i * k);
+    zd v = cconj(c.t[perm[j] * c.ldt + i]);
+    if (o.u_scale) v = cscale(v, sv[j]);
+    o.U[(long)(c.t0 + i) * k + j] = v;
+  }
 }
 
 struct __align__(16) PairSums {
@@ -472,28 +375,21 @@ __global__ void __launch_bounds__(OSJ_NT, 1) k_osj(zd* X, int m, int n, zd* T, i
         w[p] = acc;
       }
   }
-  const bool ortho = out.tall && !out.u_scale && usable;
-  bool gave_up = false;
-  if (!ortho)
-    gave_up = cb.leave();
-  else if (!cb.lost)
-    cb.sync();  // every CTA has read our sums before the rule writes over them
-  int k = 1;
-  if (!cb.lost && !gave_up) k = osj_rule(w, ws, perm, &s_k, m, out.tol, out.cap, out.gap);
-  if (ortho) {
-    if (!cb.lost)
-      k = osj_orthonormalise(c, w, ws, perm, k, f2, (zd*)part, (zd*)(part + pairs * nsub), cb, !out.r_unscale);
-    gave_up = cb.leave();
-  }
+  const bool gave_up = cb.leave();
   if (rank == 0 && tid == 0) *sweeps_out = gave_up ? -2 : converged ? max(1, sweep) : -1;
   if (gave_up) return;  // no factors
+  const int k = osj_rule(w, ws, perm, &s_k, m, out.tol, out.cap, out.gap);
   if (rank == 0 && tid == 0) *out.k_out = k;
-  osj_write(c, w, ws, perm, m, n, k, out);
+  osj_write_r(c, w, ws, perm, m, n, k, out);
+  if ((out.U == X || out.U == T) && !resident) {  // U over what R was read from: behind everyone's read
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
+  osj_write_u(c, w, perm, k, out);
 }
 
-// Row norms, rule and factors behind the rounds of separate launches.  One CTA.  coef: room for
-// 2 (m + 1) entries when U takes the rows of X.
-__global__ void __launch_bounds__(OSJ_NT) k_osj_finish(zd* X, int m, int n, zd* T, zd* coef, OsjOut out) {
+// Row norms, rule and factors behind the rounds of separate launches.  One CTA.
+__global__ void __launch_bounds__(OSJ_NT) k_osj_finish(zd* X, int m, int n, zd* T, OsjOut out) {
   extern __shared__ __align__(16) unsigned char sm[];
   double* const w = (double*)sm;
   double* const ws = w + m;
@@ -506,18 +402,12 @@ __global__ void __launch_bounds__(OSJ_NT) k_osj_finish(zd* X, int m, int n, zd* 
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) w[i] = acc;
   }
-  int k = osj_rule(w, ws, perm, &s_k, m, out.tol, out.cap, out.gap);
+  const int k = osj_rule(w, ws, perm, &s_k, m, out.tol, out.cap, out.gap);
   const OsjSlice c{X, T, n, m, 0, n, 0, m};
-  if (out.tall && !out.u_scale) {
-    double f2 = 0.0;
-    for (int i = lane; i < m; i += 32) f2 = fma(w[i], w[i], f2);
-    for (int o = 16; o > 0; o >>= 1) f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-    ClusterBarrier cb{nullptr, nullptr, 1, 0u, false};
-    if (::isfinite(f2) && f2 > 0.0)
-      k = osj_orthonormalise(c, w, ws, perm, k, f2, coef, coef + m + 1, cb, !out.r_unscale);
-  }
   if (threadIdx.x == 0) *out.k_out = k;
-  osj_write(c, w, ws, perm, m, n, k, out);
+  osj_write_r(c, w, ws, perm, m, n, k, out);
+  __syncthreads();  // U may lie over X or T
+  osj_write_u(c, w, perm, k, out);
 }
 
 // CTAs (a power of two), whether the slices fit in shared memory, and its size
@@ -581,10 +471,10 @@ cudaError_t launch_osj(zd* X, int m, int n, zd* T, int max_sweeps, int* sweeps_o
   return cudaLaunchKernelEx(&cfg, k_osj, X, m, n, T, max_sweeps, sweeps_out, (int)p.resident, out);
 }
 
-cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, zd* coef, const OsjOut& out, cudaStream_t s) {
+cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, const OsjOut& out, cudaStream_t s) {
   const size_t smem = (size_t)m * (2 * sizeof(double) + sizeof(int));
   if (smem > 48 * 1024) cudaFuncSetAttribute(k_osj_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_osj_finish<<<1, OSJ_NT, smem, s>>>(X, m, n, T, coef, out);
+  k_osj_finish<<<1, OSJ_NT, smem, s>>>(X, m, n, T, out);
   return cudaGetLastError();
 }
 

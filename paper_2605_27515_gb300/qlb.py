@@ -509,7 +509,7 @@ def qlb_svd_check(ctx: Ctx, A, tol: float = 0.0, cap: int = 0, u_scale: bool = F
     return U[:m * k.value].reshape(m, k.value), R[:k.value * n].reshape(k.value, n)
 
 
-WAIT_FACTOR, WAIT_EXCHANGE, WAIT_RANGE, WAIT_SVD = range(4)
+WAIT_FACTOR, WAIT_EXCHANGE, WAIT_RANGE, WAIT_SVD, WAIT_QR = range(5)
 
 
 def qlb_lost_wait_check(device: int, kernel: int, precision: int, n: int, cta: int):

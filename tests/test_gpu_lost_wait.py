@@ -45,3 +45,11 @@ def test_lost_wait_of_the_operator_svd(cta):
 def test_no_such_cta(kernel):
     """A CTA that has no part in a small problem holds nobody up."""
     Q.qlb_lost_wait_check(0, kernel, Q.PREC_F64, 6, 5)
+
+
+@pytest.mark.parametrize("n,cta", [(43, 0), (200, 1)])
+def test_lost_wait_of_the_qr(n, cta):
+    with pytest.raises(Q.QlbError) as e:
+        Q.qlb_lost_wait_check(0, Q.WAIT_QR, Q.PREC_F64, n, cta)
+    assert e.value.status == Q.ETIMEOUT
+    _usable(Q.PREC_F64, 64)
