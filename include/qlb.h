@@ -78,7 +78,11 @@ typedef struct {
   int device;            /* CUDA device ordinal */
   int precision;         /* QLB_PREC_* */
   double tol;            /* relative discarded-weight cutoff: keep the smallest k with
-                            sum_{i>=k} s_i^2 <= tol * sum_i s_i^2 (default 1e-12) */
+                            sum_{i>=k} s_i^2 <= tol * sum_i s_i^2 (default 1e-12).  Solves
+                            planned up to 256 rows take directions below the rounding of
+                            their Gram matrix (2^-52 of its own diagonal entry for each,
+                            2^-48 in the mixed forms) for zeros, so at tol = 0 bonds are
+                            as wide as the content that the Gram matrix resolves */
   int chi_max;           /* cap on every inter-site bond (default 64) */
   int chi_mu_max;        /* cap on the purification rank chi_mu (default 16) */
   double zip_tol_factor; /* the on-the-fly truncation inside the MPO application uses
@@ -283,9 +287,10 @@ qlb_status qlb_state_import(qlb_state* st, const void* in, size_t n_bytes);
  * one CUDA graph on the group's own stream, so n_states states cost one chain of
  * launches.  A member's numbers are the ones its own qlb_step computes: the same
  * kernels, shapes, K splits and reduction orders, bit for bit when the members
- * share one planned shape.  When planned sizes differ, an eigen-solve may run on
- * the kernel the largest co-member's size needs (the same rotations, thresholds
- * and truncation rule: results agree to rounding).  The per-class timings of
+ * share one planned shape.  When planned sizes differ, an eigen-solve or a zip-up
+ * range basis may run on the kernel the largest co-member's size needs (the same
+ * method, thresholds and truncation rule: results agree to rounding, and to the
+ * directions that `tol` above calls zeros).  The per-class timings of
  * qlb_profile_* do not cover group steps; the solver counters do.
  *
  * The members must belong to ctx, be distinct, and step the same launch sequence:

@@ -285,12 +285,12 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   *U = *Rr = nullptr;
   // A tall matrix A = Q R goes through its triangular factor: R = T^dag X by rotating its n rows,
   // so A = (Q T^dag) X with a left factor that is unitary to rounding whatever the singular values,
-  // or R^dag = T^dag X and A = (Q X^dag) T where the right factor is to be (Drmac & Veselic, "New fast and accurate Jacobi SVD algorithm I",
-  // 2008).  A sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so the tall cores of a
+  // or R^dag = T^dag X and A = (Q X^dag) T where the right factor is to be (Drmac & Veselic, "New
+  // fast and accurate Jacobi SVD algorithm I", 2008).  A sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so the tall cores of a
   // left-canonical sweep (4 D x D) cost a fortieth of rotating their own rows (admission of an
-  // N = 64 cat, 135 SVDs: 248 ms with that on one CTA, 23 now), with the same operator ranks: the
-  // rows of A^dag instead of R's left rounding in U, which the recompression took for content
-  // (transmon and resonator: bonds of 13 or 15 where 12 and 11 are).
+  // N = 64 cat, 135 SVDs: 248 ms with that on one CTA, 23 now), with the same operator ranks.
+  // Rotating the rows of A^dag leaves rounding in U that a recompression takes for content
+  // (transmon and resonator: bonds of 13 where 12 and 11 are).
   const int tall = m > n && n <= TALL_MAX_N;
   struct Buf {  // freed on return unless handed over
     qlb_ctx* c;

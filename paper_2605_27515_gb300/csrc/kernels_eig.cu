@@ -1020,8 +1020,8 @@ template <typename R>
 cudaError_t launch_eig(const EigDesc& e, const int* d_dims, cudaStream_t s, void* work, double* prof) {
   // Up to 256: pivoted Cholesky and one-sided Jacobi (kernels_pj.cu; on GB300, cold Gram
   // matrices of rank n with weights over 1e-12, best of three, against the two-sided solves
-  // here: FP64 n = 16 194 us against 698, n = 64 1.31 ms against 6.03, n = 128 4.21 ms
-  // against 38.8; double-float n = 16 102 us against 388, n = 64 0.69 ms against 3.83,
+  // here: FP64 n = 16 192 us against 698, n = 64 1.31 ms against 6.03, n = 128 4.21 ms
+  // against 38.8; double-float n = 16 100 us against 388, n = 64 0.69 ms against 3.83,
   // n = 128 2.05 ms against 23.8).  The two-sided solves stay above 256, and where they are
   // asked for as the solve of every zip-up bond: they keep directions of rounding-level
   // weight, which the pivoted factor leaves out.

@@ -6,11 +6,11 @@
 // captured as a CUDA graph.  On this GPU one SM retires ~2 FP64 FMAs per clock, so what
 // counts is how evenly the products are spread over the SMs: a 32 x 32 x 16 block of
 // complex products takes one SM 16 us, a 16 x 16 x 16 block 4 us, an 8 x 8 x 16 block 1 us.
-// The kernel is persistent over a fixed grid (at most four CTAs per SM) and decides the
-// decomposition at run time from the actual sizes: output tiles of 16 x 16 or 8 x 8 (the
-// eight warps of a CTA take a quarter of the K chunk each), whichever finishes first, or takes
-// less work in all, with its padding counted, and, with a workspace, a split of the K range into s
-// parts while tiles are fewer than CTAs and a part still outweighs what adding the parts costs.  Each
+// The kernel is persistent over a grid decided for four CTAs per SM (its registers let three
+// be resident at a time; a step launches fewer, step_gemm_ctas) and decides the decomposition
+// at run time from the actual sizes: output tiles of 16 x 16 or 8 x 8 (the eight warps of a CTA
+// take a quarter of the K chunk each), whichever finishes first, or takes less work in all, with
+// its padding counted, and, with a workspace, a split of the K range into s parts while tiles are fewer than CTAs and a part still outweighs what adding the parts costs.  Each
 // (tile, part) item writes its partial tile to the workspace; the CTA that finishes a
 // tile last (a per-tile counter, no waiting) adds the s partials in part order and applies
 // alpha and beta, so the result does not depend on timing.

@@ -36,9 +36,9 @@
 // bits, whatever larger size it was launched for; CTAs beyond C leave at once.
 //
 // Measured on GB300, cold Gram matrices of rank n with weights over 1e-12 (against the
-// two-sided Jacobi solves of kernels_eig.cu): FP64 n = 16 188 us (698), n = 32 446 us
-// (1,925), n = 64 1.28 ms (6.03), n = 128 4.14 ms (38.8); double-float n = 16 100 us (388),
-// n = 32 264 us (1,251), n = 64 0.69 ms (3.83), n = 128 2.05 ms (23.8).  At n = 64 an FP64 round of
+// two-sided Jacobi solves of kernels_eig.cu): FP64 n = 16 192 us (698), n = 32 458 us
+// (1,925), n = 64 1.31 ms (6.03), n = 128 4.21 ms (38.8); double-float n = 16 100 us (388),
+// n = 32 266 us (1,251), n = 64 0.69 ms (3.83), n = 128 2.05 ms (23.8).  At n = 64 an FP64 round of
 // four pairs to a CTA takes 4,700 cycles, ~3,500 of them the FP64 pipe; a double-float
 // round 2,100, the latency of its chain.
 //

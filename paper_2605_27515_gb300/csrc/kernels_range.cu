@@ -19,7 +19,8 @@
 //   (c) at j = cap the cut would drop real weight: the best rank-cap subspace is the top
 //       eigenvectors of G, so the kernel sets the gate and leaves the bond to the
 //       eigen-solve launched behind it (which runs only when gated in);
-//   else the column p with the largest residual norm becomes
+//   else the column p with the largest residual norm, to FP32's precision (ties go to the lower
+//   column), becomes
 //       q_j = normalise((1 - Q Q^dag) w_p)
 //   and every open column k loses its component: w_k -= q_j (q_j^dag w_k).
 //
@@ -32,8 +33,8 @@
 //
 // Measured on GB300, a cold G of rank r with weights over 1e-12 (against one CTA of 512
 // threads sweeping all columns, the kernel of the sizes above 256): FP64 n = 32, r = 16
-// 102 us (360), n = 64, r = 32 266 us (987), n = 128, r = 64 0.84 ms (4.47); double-float
-// 79 us (124), 227 us (348), 0.71 ms (2.25).  FP64 runs on four warps instead of eight, with
+// 102 us (360), n = 64, r = 32 268 us (987), n = 128, r = 64 0.85 ms (4.47); double-float
+// 81 us (124), 229 us (348), 0.72 ms (2.25).  FP64 runs on four warps instead of eight, with
 // its comparisons off the FP64 pipe (n = 64 333 us and n = 128 0.94 ms on eight): what every
 // warp computes for itself held the pipes for ~6,000 of a step's ~20,000 cycles.
 //

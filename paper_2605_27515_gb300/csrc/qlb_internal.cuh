@@ -112,11 +112,11 @@ struct GemmDesc {
   // caps on the grid (host-known maxima)
   int m_max, n_max, nb_max;
   int kclass;  // profiling class
-  // Work distribution.  Without ws: one CTA per planned output tile.  With ws (at
-  // least gemm_workspace_elems(grid) complex elements, zeroed once): a fixed grid of
-  // `grid` CTAs (0 = four per SM) that splits the K range at run time so that tiles x
-  // parts fill it; ksplit >= 1 caps that split (0: the default cap).  The last CTA of a tile adds the
-  // partials in part order (deterministic).
+  // Work distribution.  Without ws: no K split, a CTA per planned tile of 8 x 8 up to `grid`
+  // CTAs, each taking tiles in turn.  With ws (at least gemm_workspace_elems(grid) complex
+  // elements, zeroed once): a fixed grid of `grid` CTAs (0 = four per SM) that splits the K
+  // range at run time so that tiles x parts fill it; ksplit >= 1 caps that split (0: the
+  // default cap).  The last CTA of a tile adds the partials in part order (deterministic).
   int ksplit;
   void* ws;
   int grid;
