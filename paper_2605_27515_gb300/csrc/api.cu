@@ -1182,8 +1182,7 @@ static qlb_status svd_lost_wait(int device, int n, const std::vector<double>& M,
   int h = 0;
   cudaError_t e = cudaMemcpy(buf, M.data(), sizeof(zd) * 4 * nn, cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
-    e = qr ? launch_tall_qr(buf, 4 * n, n, 0, buf + 4 * nn, buf + 5 * nn, (double*)(buf + 6 * nn), d_out, d_out + 1,
-                            cta + 1, 0)
+    e = qr ? launch_tall_qr(buf, 4 * n, n, 0, buf + 4 * nn, d_out, d_out + 1, cta + 1, 0)
            : launch_osj(buf, n, 4 * n, buf + 4 * nn, 60, d_out, out, 0);
   if (e == cudaSuccess) e = cudaMemcpy(&h, d_out, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(buf);

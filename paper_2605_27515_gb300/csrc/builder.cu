@@ -284,11 +284,11 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   cudaStream_t s = ctx->stream;
   *U = *Rr = nullptr;
   // A tall matrix A = Q R goes through its triangular factor: R = T^dag X by rotating its n rows,
-  // so A = (Q T^dag) X with a left factor that is unitary to rounding whatever the singular values,
-  // or R^dag = T^dag X and A = (Q X^dag) T where the right factor is to be (Drmac & Veselic, "New
-  // fast and accurate Jacobi SVD algorithm I", 2008).  A sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so the tall cores of a
+  // so A = (Q T^dag) X with a left factor that is orthonormal to rounding whatever the singular
+  // values, or R^dag = T^dag X and A = (Q X^dag) T where the right factor is to be (Drmac & Veselic,
+  // "New fast and accurate Jacobi SVD algorithm I", 2008).  A sweep takes rows^2 / 2 pairs of ~20 (rows + columns) FMAs, so the tall cores of a
   // left-canonical sweep (4 D x D) cost a fortieth of rotating their own rows (admission of an
-  // N = 64 cat, 135 SVDs: 248 ms with that on one CTA, 23 now), with the same operator ranks.
+  // N = 64 cat, 135 SVDs: 248 ms with that on one CTA, 22 now), with the same operator ranks.
   // Rotating the rows of A^dag leaves rounding in U that a recompression takes for content
   // (transmon and resonator: bonds of 13 where 12 and 11 are).
   const int tall = m > n && n <= TALL_MAX_N;
@@ -304,21 +304,18 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   qlb_status st;
   const int rows = tall ? n : m;  // rotated; the factors are at most that wide
   const size_t r2 = sizeof(zd) * (size_t)rows * rows;
-  // counts, then the heads and factors of the reflectors
-  if ((st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double) + (tall ? (sizeof(zd) + sizeof(double)) * (size_t)n : 0))) ||
+  if ((st = dev_alloc_queued(ctx, &bc.p, 4 * sizeof(double))) ||
       (st = dev_alloc_queued(ctx, &bt.p, r2)) || (tall && (st = dev_alloc_queued(ctx, &bx.p, r2))) ||
       (!tall && (st = dev_alloc_queued(ctx, &bu.p, r2))) ||
       (st = dev_alloc_queued(ctx, &br.p, sizeof(zd) * (size_t)rows * n)))
     return st;
   // sweeps or rotations, kept count, (a threshold,) [4] status of the QR
   int* d_cnt = (int*)bc.p;
-  zd* const v0 = (zd*)((double*)bc.p + 4);
-  double* const tau = (double*)(v0 + n);
   zd *const A = X, *const T = (zd*)bt.p;
   const int am = m, dagger = tall && u_scale && r_unscale;
   if (tall) {
     X = (zd*)bx.p;
-    QLB_CUDA_TRY(launch_tall_qr(A, m, n, dagger, X, v0, tau, d_cnt + 4, d_cnt + 1, 0, s));
+    QLB_CUDA_TRY(launch_tall_qr(A, m, n, dagger, X, d_cnt + 4, d_cnt + 1, 0, s));
     m = n;
   }
   zd* const small_u = dagger ? T : X;  // U of R, over what the right factor has been read from
@@ -350,7 +347,21 @@ qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** 
   if (tall) {
     (dagger ? bx : bt).release();  // (in the stream's order) so that U takes no more than rotating A's own rows did
     if ((st = dev_alloc_queued(ctx, &bu.p, sizeof(zd) * (size_t)am * n))) return st;
-    QLB_CUDA_TRY(launch_tall_apply(A, am, n, v0, tau, small_u, d_cnt + 1, (zd*)bu.p, s));
+    GemmDesc g{};
+    g.A = A;
+    g.B = small_u;
+    g.C = bu.p;
+    g.m = dconst(am);
+    g.n = g.ldb = g.ldc = dvar(1);  // the kept count
+    g.k = g.lda = dconst(n);
+    g.sA1 = g.sB1 = g.sC1 = g.sA2 = g.sB2 = g.sC2 = dconst(0);
+    g.nb1 = g.nb2 = dconst(1);
+    g.opA = g.opB = OP_N;
+    g.alpha_re = 1;
+    g.m_max = am;
+    g.n_max = n;
+    g.nb_max = 1;
+    QLB_CUDA_TRY(launch_gemm(g, d_cnt, s, nullptr));
   }
   cudaMemcpyAsync(h, d_cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);

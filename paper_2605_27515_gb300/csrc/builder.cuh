@@ -84,14 +84,10 @@ cudaError_t launch_osj(zd* X, int m, int n, zd* T, int max_sweeps, int* sweeps_o
 cudaError_t launch_osj_finish(zd* X, int m, int n, zd* T, const OsjOut& out, cudaStream_t s);
 // columns of a tall matrix that goes through its QR (kernels_tallqr.cu: its rows' buffers)
 constexpr int TALL_MAX_N = 2048;
-// Householder QR of a tall matrix (kernels_tallqr.cu): A (m x n, m > n) becomes the reflectors
-// (below the diagonal; their heads v0 and factors tau aside) and R, or R^dag if dagger (n x n).
-// *status: 0, or -2 when a bounded wait gave up; *count: 0.  stall as in OsjOut.
-cudaError_t launch_tall_qr(zd* A, int m, int n, int dagger, zd* R, zd* v0, double* tau, int* status, int* count,
-                           int stall, cudaStream_t s);
-// U (m x k) = Q C for C of n x k, k read from device memory
-cudaError_t launch_tall_apply(const zd* A, int m, int n, const zd* v0, const double* tau, const zd* C, const int* k,
-                              zd* U, cudaStream_t s);
+// QR of a tall matrix (kernels_tallqr.cu): A (m x n, m > n) becomes Q; R, or R^dag if dagger, n x n.
+// Columns without a new direction are zero in Q, their rows zero in R.  *status: 0, or -2 when a
+// bounded wait gave up; *count: 0.  stall as in OsjOut.
+cudaError_t launch_tall_qr(zd* A, int m, int n, int dagger, zd* R, int* status, int* count, int stall, cudaStream_t s);
 void init_tallqr_attributes();
 void init_osj_attributes();
 qlb_status svd_osj(qlb_ctx* ctx, zd* X, int m, int n, double tol, int cap, zd** U, int u_scale, zd** Rr,

@@ -137,3 +137,15 @@ def test_operator_ranks():
     assert b.ops["H0"].bond_dims() == [4, 5, 5, 5, 5, 5, 3, 6, 8, 12, 12, 12, 12, 11, 7, 4]
     assert b.ops["H1"].bond_dims() == [1, 1, 1, 1, 1, 1, 1, 4, 6, 10, 11, 11, 11, 9, 5, 2]
     c.close()
+
+
+@pytest.mark.parametrize("R", [3, 6, 9])
+def test_far_levels_stay_uncoupled(R):
+    """a^2 - alpha^2 couples levels n and n - 2 only: every other off-diagonal entry of its MPO is an
+    exact zero, as the supports of the cores' rows do not meet."""
+    c = Q.Ctx(device=0)
+    s = Q.System(c, [R])
+    D = s.op([(1.0, [(0, Q.F_A, 2)]), (-16.0, [])]).to_dense()
+    i, j = np.indices(D.shape)
+    assert np.count_nonzero(D[(i != j) & (j != i + 2)]) == 0
+    c.close()
